@@ -204,7 +204,7 @@ class Pipeline:
                 fn()
             self.graphs.append(gr)
         # the whole step: the gradient zeroing runs on a branch of the graph forked after the
-        # projection, concurrently with the sort (whose passes leave most SMs idle) and the
+        # projection, concurrently with the sort (whose launches leave most SMs idle) and the
         # forward, and joined before the backward (a zeroing still running beside the persistent
         # compositing adjoint would wait for free SMs)
         self.whole = torch.cuda.CUDAGraph()
@@ -876,13 +876,12 @@ def main():
     P, K = pipe.pb.P, stats["num_keys"]
     wsv = pipe.pb.workspace()
     passes, G = wsv["passes"], wsv["tile_ranges"].shape[0]
-    onesweep = pipe.pb.params.sort_mode == R.L.GS_SORT_ONESWEEP
-    vis = int((wsv["tiles_touched"] != 0).sum().item()) if not onesweep else 0
     npx = pipe.V * pipe.pb.W * pipe.pb.H
     alg_bytes = {
         "project": P * 60 + 0,
-        "bin_sort": (P * 8 + K * 12 + passes * K * 24 + K * 8 + G * 8) if onesweep else
-                    (G * 8 + vis * 32 + K * 12 + K * 116),
+        # tile-first: inclusive sums, tile counts and ranges, 48 B per key through the slices, its record read,
+        # and key, value and record written
+        "bin_sort": P * 8 + G * 20 + K * 156,
         "render_fwd_l1": npx * 48,
         "project_bwd": P * 60,
         "pose_grad": 0,

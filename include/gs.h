@@ -69,16 +69,16 @@ typedef struct gs_camera {
 
 /* Binning algorithms of gs_bin_sort.  Both produce the same lists bit for bit: every tile's
  * entries ordered by (depth bits, flattened pair index).
- *   GS_SORT_ONESWEEP (default): scan of tiles_touched, keys (tile << 32 | depth bits) in emission
- *     order and the digit histograms of every pass (one kernel), then a stable LSD onesweep radix
- *     sort over all keys (8-bit digits, decoupled look-back).
- *   GS_SORT_TILE_BUCKET: gs_project counts the keys of every tile, a scan of the G counts gives
- *     each tile its slice, emission drops each key into its tile's slice by atomic slot taking
- *     (order inside the slice arbitrary), and each tile's slice is sorted by (depth bits, pair
- *     index) in shared memory (a warp per slice of at most 128 entries, a CTA per longer slice,
- *     slices longer than 4096 entries as sorted runs merged in global memory).  No global sort,
- *     but one atomic per key twice; measured slower than the onesweep path on GB300 except for
- *     small single-view problems. */
+ *   Tile-first: the keys of every tile are counted, a scan of the G counts gives each tile its slice,
+ *     every key is dropped into its slice as the word (depth bits, pair index) in arbitrary order and
+ *     each slice is sorted on chip (a warp per slice of at most 256 words, a CTA per longer one, slices
+ *     longer than 4096 words as sorted runs merged in global memory).  Faster for few or short lists.
+ *   Radix: the visible pairs sorted by depth, their keys emitted in that order and sorted by tile, both
+ *     by a stable LSD onesweep radix sort (at most 8-bit digits, decoupled look-back).  Faster for many
+ *     long lists.
+ * GS_SORT_TILE_BUCKET always takes the tile-first binning and leaves tiles_touched as counts;
+ * GS_SORT_ONESWEEP (default) takes whichever suits the problem's size and leaves tiles_touched as
+ * inclusive sums. */
 enum { GS_SORT_TILE_BUCKET = 0, GS_SORT_ONESWEEP = 1 };
 
 /* Rasterizer constants.  gs_default_params() gives tile 16x16, near 0.2, dilation 0.3,
@@ -165,7 +165,7 @@ typedef struct gs_ws_view {
     uint32_t *num_keys;
     int64_t num_pairs;                 /* P */
     int64_t num_tiles;                 /* G */
-    int32_t sort_passes;               /* 8-bit LSD passes of the onesweep sort */
+    int32_t sort_passes;               /* LSD passes of the radix binning (4 over the depth, then the tile) */
     int32_t reserved;
     uint32_t *pair_slot;               /* [P] slot of each visible pair, 0xffffffff if culled */
     int64_t visible_capacity;          /* slots in proj and grad2d */
@@ -220,7 +220,7 @@ int gs_read_stats(const gs_problem *pb, void *ws, void *stream, gs_stats *out);
 /* Workspace guard blocks (no counterpart in the paper; a check of the library itself): 256-byte
  * blocks of a fixed byte pattern, written by gs_workspace_init, follow every workspace buffer that
  * kernels index with data (projection records, tile counts, both key and value buffers, the tile
- * ranges and lists, the records in list order, the 2-D gradients, the pose partials, the pair
+ * ranges, the emission's work items, the records in list order, the 2-D gradients, the pose partials, the pair
  * slots, the claim-class lists).  This call
  * synchronises `stream` and returns GS_OK when every block is intact, else GS_ERR_DEVICE_FAULT with
  * *first_bad (may be NULL) = the index of the first changed block in that order. */
@@ -235,8 +235,7 @@ int32_t gs_checked_build(void);
 
 /* EWA projection of every (view, Gaussian) pair (Eq. 19 covariance form, world-to-camera poses
  * of Eq. 15): camera transform, 2-D conic with dilation, radius, tile rectangle, touched-tile
- * count; writes proj and tiles_touched in the workspace (and, with GS_SORT_TILE_BUCKET, the key
- * count of every tile). */
+ * count; writes proj and tiles_touched in the workspace. */
 int gs_project(const gs_problem *pb, const gs_gaussians *g, void *ws, void *stream);
 
 /* Tile binning (params.sort_mode selects the algorithm, see GS_SORT_*): per-tile lists ordered by

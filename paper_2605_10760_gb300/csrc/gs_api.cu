@@ -89,8 +89,10 @@ int compute_layout(const gs_problem *pb, Layout *L) {
     while ((1LL << gbits) < L->G) ++gbits;
     L->passes = (32 + gbits + 7) / 8;
     if (L->passes > kMaxPasses) return GS_ERR_INVALID_ARG;
-    // the scan runs over the P touched-tile counts (onesweep) or the G tile key counts (bucket)
-    L->scan_parts = std::max<long long>(1, (std::max(P, L->G) + kScanTile - 1) / kScanTile);
+    L->tile_passes = (gbits + 7) / 8;          // the passes above the four over the depth, their bits split evenly
+    L->tile_bits = L->tile_passes > 0 ? (gbits + L->tile_passes - 1) / L->tile_passes : 0;
+    // the scan runs over the P touched-tile counts (onesweep) or the chunks' key counts (tile-first)
+    L->scan_parts = std::max<long long>(1, (P + kScanTile - 1) / kScanTile);
     const long long sort_tile = (long long)kSortThreads * kSortIPT;
     L->sort_parts = std::max<long long>(1, (L->cap + sort_tile - 1) / sort_tile);
     long long chunks_total = 0;
@@ -111,15 +113,19 @@ int compute_layout(const gs_problem *pb, Layout *L) {
     guard();
     for (int k = 0; k < 2; ++k) { L->o_keys[k] = o; o = align256(o + sizeof(uint64_t) * (size_t)L->cap); guard(); }
     for (int k = 0; k < 2; ++k) { L->o_vals[k] = o; o = align256(o + sizeof(uint32_t) * (size_t)L->cap); guard(); }
-    // scan_state .. ranges are adjacent: the onesweep binning clears them with one memset
+    // adjacent spans, each cleared with one memset: tcnt .. scan_state before the tile-first binning,
+    // scan_state .. ranges before the radix binning
+    L->o_tcnt = o; o = align256(o + sizeof(uint32_t) * (size_t)L->G);
+    L->o_tscan = o; o = align256(o + sizeof(unsigned long long) * (size_t)((L->G + kScanTile - 1) / kScanTile));
     L->o_scan_state = o; o = align256(o + sizeof(unsigned long long) * L->scan_parts);
+    L->o_vscan = o; o = align256(o + sizeof(unsigned long long) * L->scan_parts);
+    const long long emit_pairs = std::max<long long>(1, std::min(L->cap, P));
+    L->o_escan = o; o = align256(o + sizeof(unsigned long long) * (size_t)((emit_pairs + kEmitPart - 1) / kEmitPart));
     L->o_hist = o; o = align256(o + sizeof(uint32_t) * kMaxPasses * 256);
     L->o_sort_state = o; o = align256(o + sizeof(uint32_t) * 256 * (size_t)L->sort_parts * L->passes);
     L->o_ranges = o; o = align256(o + sizeof(uint32_t) * 2 * (size_t)L->G);
-    L->o_tword = o; o = align256(o + sizeof(unsigned long long) * (size_t)L->G);
     guard();
-    L->o_tcnt = o; o = align256(o + sizeof(uint32_t) * ((size_t)L->G + 1) + 64);
-    L->o_tlist = o; o = align256(o + sizeof(uint32_t) * (size_t)L->G);
+    L->o_extra = o; o = align256(o + sizeof(uint2) * (size_t)(L->cap / kEmitKeysMin + 1));
     guard();
     L->o_srec = o; o = align256(o + sizeof(float) * 12 * (size_t)L->cap);
     guard();
@@ -356,10 +362,6 @@ int gs_project(const gs_problem *pb, const gs_gaussians *g, void *ws, void *stre
     if (!ws_ok(ws) || !g || !pb->cameras) return GS_ERR_INVALID_ARG;
     if (L.N > 0 && (!g->means || !g->log_scales || !g->quats || !g->opacities || !g->colors)) return GS_ERR_INVALID_ARG;
     if (((uintptr_t)g->quats & 15) != 0) return GS_ERR_INVALID_ARG;
-    if (L.sort_mode == GS_SORT_TILE_BUCKET &&
-        cudaMemsetAsync(ws_ptr<uint32_t>(ws, L.o_tcnt), 0, sizeof(uint32_t) * ((size_t)L.G + 1),
-                        (cudaStream_t)stream) != cudaSuccess)
-        return GS_ERR_CUDA;
     DevStatus *st = ws_ptr<DevStatus>(ws, L.o_status);
     if (L.P == 0)   // no projection launch: no slots taken
         return cudaMemsetAsync(&st->num_visible, 0, sizeof(st->num_visible), (cudaStream_t)stream) == cudaSuccess
@@ -375,7 +377,6 @@ int gs_project(const gs_problem *pb, const gs_gaussians *g, void *ws, void *stre
     a.itw = 1.0f / (float)L.tw; a.ith = 1.0f / (float)L.th; a.Tx = (float)L.Tx; a.Ty = (float)L.Ty;
     a.near_plane = pb->params.near_plane; a.dil = pb->params.dilation; a.sigmas = pb->params.radius_sigmas;
     a.alpha_min = pb->params.alpha_min;
-    a.tile_cnt = L.sort_mode == GS_SORT_TILE_BUCKET ? ws_ptr<uint32_t>(ws, L.o_tcnt) : nullptr;
     a.P = L.P;
     a.st = st;
     a.slot = ws_ptr<uint32_t>(ws, L.o_slot);
@@ -383,8 +384,6 @@ int gs_project(const gs_problem *pb, const gs_gaussians *g, void *ws, void *stre
     a.slane = ws_ptr<uint16_t>(ws, L.o_slane);
     a.blk = ws_ptr<uint4>(ws, L.o_blk);
     a.chunks = L.chunks_total;
-    a.Txi = L.Tx;
-    a.Ty_i = L.Ty;
     launch_project(L, a, (cudaStream_t)stream);
     return check_launch();
 }
@@ -408,18 +407,44 @@ static BinArgs make_bin_args(const Layout &L, void *ws) {
     a.st = ws_ptr<DevStatus>(ws, L.o_status);
     a.V = L.V; a.Tx = L.Tx; a.Ty = L.Ty; a.passes = L.passes;
     a.itw = 1.0f / (float)L.tw; a.ith = 1.0f / (float)L.th;
-    a.P = L.P; a.cap = L.cap; a.sort_parts = L.sort_parts; a.max_chunks = L.max_chunks; a.G = L.G;
+    a.P = L.P; a.cap = L.cap; a.sort_parts = L.sort_parts; a.G = L.G; a.max_count = L.max_count;
     a.slot = ws_ptr<const uint32_t>(ws, L.o_slot);
     a.vcap = L.vcap;
     a.fault_scan_part = -1;
     a.spin_limit = kSpinLimit;
     a.sort_mode = L.sort_mode;
+    if (a.sort_mode == GS_SORT_TILE_BUCKET) a.touched = nullptr;   // this mode leaves the counts
+    a.blk = ws_ptr<uint4>(ws, L.o_blk);
+    a.slane = ws_ptr<const uint16_t>(ws, L.o_slane);
+    a.chunks = L.chunks_total;
     a.tile_cnt = ws_ptr<uint32_t>(ws, L.o_tcnt);
-    a.tile_list = ws_ptr<uint32_t>(ws, L.o_tlist);
-    a.tword = ws_ptr<unsigned long long>(ws, L.o_tword);
+    a.tile_scan_state = ws_ptr<unsigned long long>(ws, L.o_tscan);
+    a.items = ws_ptr<uint4>(ws, L.o_srec);
+    a.words = ws_ptr<unsigned long long>(ws, L.o_keys[(L.passes & 1) ^ 1]);
+    a.extra = ws_ptr<uint2>(ws, L.o_extra);
+    a.extra_cap = (uint32_t)(L.cap / kEmitKeysMin + 1);
+    a.bucket_clear_begin = ws_ptr<unsigned char>(ws, L.o_tcnt);
+    a.bucket_clear_bytes = L.o_vscan - L.o_tcnt;
+    // radix binning: the pairs' arrays and one half of the keys' ping-pong lie in the records' buffer (written
+    // last), the other half, where the last pass ends, in the key buffer that is not the output
+    a.vis_scan_state = ws_ptr<unsigned long long>(ws, L.o_vscan);
+    a.emit_scan_state = ws_ptr<unsigned long long>(ws, L.o_escan);
+    const size_t quarter = sizeof(uint32_t) * (size_t)L.cap;
+    for (int k = 0; k < 2; ++k) {
+        a.pkey[k] = ws_ptr<uint32_t>(ws, L.o_srec + quarter * (2 * k));
+        a.pval[k] = ws_ptr<uint32_t>(ws, L.o_srec + quarter * (2 * k + 1));
+    }
+    a.info = ws_ptr<uint4>(ws, L.o_srec + 4 * quarter);
+    a.tile_passes = L.tile_passes;
+    a.tile_bits = L.tile_bits;
+    const int last = L.tile_passes & 1;
+    a.tkey[last] = ws_ptr<uint32_t>(ws, L.o_keys[(L.passes & 1) ^ 1]);
+    a.tval[last] = a.tkey[last] + L.cap;
+    a.tkey[last ^ 1] = ws_ptr<uint32_t>(ws, L.o_srec + 8 * quarter);
+    a.tval[last ^ 1] = a.tkey[last ^ 1] + L.cap;
     a.clist = ws_ptr<uint32_t>(ws, L.o_clist);
     a.clear_begin = ws_ptr<unsigned char>(ws, L.o_scan_state);
-    a.clear_bytes = L.o_tword + sizeof(unsigned long long) * (size_t)L.G - L.o_scan_state;
+    a.clear_bytes = L.o_ranges + sizeof(uint32_t) * 2 * (size_t)L.G - L.o_scan_state;
     return a;
 }
 

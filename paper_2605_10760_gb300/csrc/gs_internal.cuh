@@ -24,11 +24,14 @@ constexpr int kScanThreads = 256;
 constexpr int kScanIPT = 16;
 constexpr int kScanTile = kScanThreads * kScanIPT;
 constexpr int kChunk = 256;            // (view, Gaussian) pairs per projection block
+constexpr int kEmitPart = 1024;        // pairs per partition of the depth-ordered emission
+constexpr int kMaxTilePasses = 4;
+constexpr uint32_t kEmitKeysMin = 512; // keys per work item of the tile-first emission, at the least
 constexpr unsigned long long kSpinLimit = 1ull << 21;  // bounded waits (x ~100 ns sleep)
 
-// counters inside the status block (zeroed by the call that uses them)
+// counters inside the status block (zero between calls: every launch returns its own to zero)
 enum Counter {
-    kCtrScan = 0, kCtrSort0 = 1, kCtrTileSort = 14, kCtrTileList = 15, kCtrTileLong = 16,
+    kCtrScan = 0, kCtrSort0 = 1, kCtrTileScan = 14, kCtrEmitExtra = 15, kCtrEmitSorted = 16,
     kNumCounters = 32
 };
 
@@ -52,7 +55,17 @@ struct DevStatus {
     // the projection's slot counter: blocks that have reserved << 40 | slots reserved; the block
     // arriving last publishes num_visible and returns it to zero
     unsigned long long slot_ctr;
+    unsigned long long bin_pairs;     // visible pairs of the radix binning
 };
+
+// a projection block's counts: candidates (slots taken), visible pairs, view (< GS_MAX_VIEWS = 1024)
+__host__ __device__ inline uint32_t blk_pack(uint32_t candidates, uint32_t visible, uint32_t view) {
+    return candidates | (visible << 9) | (view << 18);
+}
+__host__ __device__ inline uint32_t blk_candidates(uint32_t y) { return y & 511u; }
+__host__ __device__ inline uint32_t blk_visible(uint32_t y) { return (y >> 9) & 511u; }
+__host__ __device__ inline int blk_view(uint32_t y) { return (int)(y >> 18); }
+static_assert(kChunk <= 511 && GS_MAX_VIEWS <= 1 << 14, "fields of blk_pack");
 
 struct ViewEntry {                // per-view table in the workspace (32 bytes)
     long long gauss_begin;
@@ -64,16 +77,16 @@ struct ViewEntry {                // per-view table in the workspace (32 bytes)
 constexpr int kNumGuards = 15;
 
 struct Layout {
-    int V, W, H, tw, th, Tx, Ty, passes;
+    int V, W, H, tw, th, Tx, Ty, passes, tile_passes, tile_bits;
     long long G, P, N, cap, max_count, max_chunks;
     long long vcap;                    // slots of the projection records and 2-D gradients
     long long scan_parts, sort_parts, chunks_total;
     int sort_mode, nb;                 // binning mode; records per staged render batch
     size_t o_status, o_views, o_proj, o_touched, o_scan_state, o_keys[2], o_vals[2], o_hist,
-        o_sort_state, o_ranges, o_tword, o_tcnt, o_tlist, o_srec, o_g2d, o_pose_part, o_slot, o_clist, o_slane,
+        o_sort_state, o_ranges, o_tcnt, o_tscan, o_vscan, o_escan, o_extra, o_srec, o_g2d, o_pose_part, o_slot, o_clist, o_slane,
         o_blk, total;
     size_t o_guard[kNumGuards];        // guard blocks after proj, touched, keys x2, vals x2, ranges,
-                                       // the tile lists, srec, g2d, the pose partials, the slots,
+                                       // the extra emission items, srec, g2d, the pose partials, the slots,
                                        // the claim-class lists, the slot lanes, the block slot ranges
 };
 constexpr uint32_t kNoSlot = 0xffffffffu;   // pair_slot of a culled pair
@@ -329,6 +342,37 @@ __device__ __forceinline__ unsigned lanemask_lt() {
     return m;
 }
 
+
+// ------------------------------------------------------------------------------------------
+// claim order of the work items
+// ------------------------------------------------------------------------------------------
+// Claim order: the binning lists every (view, tile) item under its claim class (class 0 the
+// longest lists); coff[k] is the number of items in classes below k (coff[kClaimClasses] = all),
+// so the counter's value c falls in the class k with coff[k] <= c < coff[k + 1].
+__device__ __forceinline__ void claim_offsets(const DevStatus *st, uint32_t *coff) {
+    if (threadIdx.x < 32) {
+        static_assert(kClaimClasses == 32, "one class per lane");
+        const uint32_t x = st->claim_cnt[threadIdx.x];
+        uint32_t y = x;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(0xffffffffu, y, o);
+            if ((int)threadIdx.x >= o) y += t;
+        }
+        coff[threadIdx.x] = y - x;
+        if (threadIdx.x == 31) coff[32] = y;
+    }
+}
+
+// Item number c of the claim order (2^32 - 1 or more when the class lists are inconsistent).
+__device__ __forceinline__ long long claim_at(const uint32_t *coff, const uint32_t *clist, long long G, long long c) {
+    int k = 0;   // the largest k with coff[k] <= c (coff[0] = 0)
+#pragma unroll
+    for (int step = kClaimClasses / 2; step > 0; step >>= 1)
+        if ((long long)coff[k + step] <= c) k += step;
+    const long long r = c - (long long)coff[k];
+    return r < G ? (long long)clist[(size_t)k * G + r] : 0xffffffffLL;
+}
 
 // ------------------------------------------------------------------------------------------
 // TMA bulk copies (cp.async.bulk, 1-D) completing on shared-memory mbarriers

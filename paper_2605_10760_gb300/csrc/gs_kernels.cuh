@@ -15,15 +15,14 @@ struct ProjArgs {
     int W, H;
     float itw, ith, Tx, Ty;     // 1 / tile size (exact: tile sizes are powers of two), tiles per row / column
     float near_plane, dil, sigmas, alpha_min;
-    uint32_t *tile_cnt;         // [G] key count per global tile (tile-bucket binning), else null
-    int Txi, Ty_i;
     long long P;                // (view, Gaussian) pairs: the length of touched and slot
     DevStatus *st;              // errors; slot_ctr hands out the slots, num_visible their count
     uint32_t *slot;             // [P] slot of each visible pair in proj (kNoSlot when culled)
     long long vcap;             // slots in proj
     uint16_t *slane;            // [vcap] the chunk position of each slot's pair, | kSlotHole when the
                                 //   decision chain culled it
-    uint4 *blk;                 // [chunks] first slot and candidate count of each projection block
+    uint4 *blk;                 // [chunks] of each projection block: first slot, blk_pack() word, key count, and
+                                //   room for the binning's key offset
     long long chunks;           // projection blocks over all views (the length of blk)
 };
 
@@ -52,7 +51,7 @@ void launch_pose_reduce(const Layout &L, const ViewEntry *views, const float *pa
 // ---------------- binning ----------------
 struct BinArgs {
     const ViewEntry *views;
-    uint32_t *touched;                 // in: counts; out: inclusive prefix sums
+    uint32_t *touched;                 // in: counts; out: inclusive prefix sums (null: the counts stay)
     unsigned long long *scan_state;
     const float4 *proj;
     float4 *g2d;
@@ -65,24 +64,46 @@ struct BinArgs {
     DevStatus *st;
     int V, Tx, Ty, passes;
     float itw, ith;                    // 1 / tile size (exact: tile sizes are powers of two)
-    long long P, cap, sort_parts, max_chunks, G;
+    long long P, cap, sort_parts, G, max_count;   // max_count: Gaussians of the largest view
     int fault_scan_part;               // -1 normally; >= 0: that scan partition never publishes
-    void *clear_begin;                 // scan_state, hist, sort_state and ranges: one span cleared before
-    size_t clear_bytes;                //   the onesweep binning
+    void *clear_begin;                 // scan_state .. ranges: one span cleared before the radix binning
+    size_t clear_bytes;
+    void *bucket_clear_begin;          // tile_cnt, tile_scan_state and scan_state: one span cleared before
+    size_t bucket_clear_bytes;         //   the tile-first binning
     unsigned long long spin_limit;
     int sort_mode;                     // GS_SORT_TILE_BUCKET or GS_SORT_ONESWEEP
-    uint32_t *tile_cnt;                // [G + 1] per-tile key counts -> slice starts (bucket mode)
-    uint32_t *tile_list;               // [G] tiles whose slices are sorted by k_tile_sort_long
     const uint32_t *slot;              // [P] slot of each visible pair in proj and g2d
     long long vcap;                    // slots in proj and g2d
-    unsigned long long *tword;         // [G] start/end combining words of the ranges kernel
+    // radix binning
+    unsigned long long *vis_scan_state, *emit_scan_state;   // [chunk partitions], [partitions of kEmitPart pairs]
+    uint32_t *pkey[2], *pval[2];       // [cap] depth bits and position of each visible pair, ping-pong
+    uint4 *info;                       // [cap] by position: first tile, rectangle width, key count, pair
+    uint32_t *tkey[2], *tval[2];       // [cap] tile and pair of each key, ping-pong
+    int tile_passes, tile_bits;        // radix passes over the tile and bits of each
+    // tile-first binning
+    uint4 *blk;                        // [chunks] the projection blocks (key count in z, key offset out in w)
+    const uint16_t *slane;             // [vcap] chunk position of each slot's pair (| kSlotHole: a hole)
+    long long chunks;
+    uint32_t *tile_cnt;                // [G] keys per tile
+    unsigned long long *tile_scan_state;
+    uint4 *items;                      // [K] (tile, rank in tile, depth bits, pair): the records' buffer before
+                                       //   they are written
+    unsigned long long *words;         // [K] (depth bits << 32 | pair) in the tiles' slices: the key buffer that is
+                                       //   not the output
+    uint2 *extra;                      // [extra_cap] further (chunk, portion) items of the emission
+    uint32_t extra_cap, emit_keys;     // keys per emission item
+    long long long_blocks;             // CTAs of the sort that take the long lists
     uint32_t *clist;                   // [kClaimClasses, G] out: the items of each claim class
 };
 
-// onesweep: scan with key emission and digit histograms -> onesweep passes -> ranges; tile bucket: scan of the
-// tile counts -> emission into tile slices -> per-tile sort.  Either way the sorted keys end in
-// keys[passes % 2], the values in vals[passes % 2], the records in list order in srec
+// Either way the sorted keys end in keys[passes % 2], the values in vals[passes % 2], the records in
+// list order in srec.  run_bin_sort chooses: tile-first (gs_bin.cu: keys into tile slices, every slice
+// sorted on chip) or run_onesweep (gs_sort.cu: scan with key emission and digit histograms -> onesweep
+// passes -> ranges).
 int run_bin_sort(const BinArgs &a, cudaStream_t s);
+int run_onesweep(const BinArgs &a, cudaStream_t s);
+void launch_scan_chunks(const BinArgs &a, bool pairs, cudaStream_t s);
+void launch_claims(const BinArgs &a, cudaStream_t s);
 // scan alone (used by the bounded-wait test entry point)
 int run_scan_only(const BinArgs &a, cudaStream_t s);
 

@@ -126,6 +126,7 @@ __global__ void __launch_bounds__(kProjThreads) k_project(ProjArgs a) {
         }
     }
     // phase 2: candidates r kProjThreads + thread through the decision chain
+    uint32_t keys = 0, nvis = 0;  // touched tiles and visible pairs of this thread
     const int rounds = (int)((ncand + kProjThreads - 1) / kProjThreads);
     for (int r = 0; r < rounds; ++r) {
         const int t = r * kProjThreads + threadIdx.x;
@@ -179,17 +180,27 @@ __global__ void __launch_bounds__(kProjThreads) k_project(ProjArgs a) {
                 rec[2] = make_float4(c0, c1, c2, cut);
             }
             a.touched[f] = cnt;
-        }
-        if (a.tile_cnt && o.visible) {   // tile-bucket binning: one key per touched tile of this view
-            uint32_t *row = a.tile_cnt + (size_t)v * a.Txi * a.Ty_i;
-            for (int ty = o.y0; ty < o.y1; ++ty)
-                for (int tx = o.x0; tx < o.x1; ++tx) atomicAdd(row + ty * a.Txi + tx, 1u);
+            keys += cnt;
+            nvis += o.visible ? 1u : 0u;
         }
     }
+    keys = __reduce_add_sync(0xffffffffu, keys);   // (s_wcnt was last read before the barrier above)
+    nvis = __reduce_add_sync(0xffffffffu, nvis);
+    static_assert(kProjPre >= 2, "two rows of s_wcnt");
+    if (lane == 0) {
+        s_wcnt[0][warp] = keys;
+        s_wcnt[1][warp] = nvis;
+    }
+    __syncthreads();
     if (threadIdx.x == 0) {
         const long long ch = s_ve.chunk_off + blockIdx.x;
+        uint32_t total = 0, vis = 0;
+        for (int w = 0; w < kProjThreads / 32; ++w) {
+            total += s_wcnt[0][w];
+            vis += s_wcnt[1][w];
+        }
         if (base_i < s_ve.count && gs_guard(a.st, ch < a.chunks, 6))
-            a.blk[ch] = make_uint4((uint32_t)min(base_reg, (unsigned long long)a.vcap), ncand, 0u, 0u);
+            a.blk[ch] = make_uint4((uint32_t)min(base_reg, (unsigned long long)a.vcap), blk_pack(ncand, vis, (uint32_t)v), total, 0u);
     }
 }
 
@@ -239,7 +250,7 @@ __global__ void __launch_bounds__(kProjBwdThreads, 16) k_project_bwd(ProjBwdArgs
     // projection); holes (candidates the decision chain culled) are flagged in their slot lane
     const unsigned long long vc = (unsigned long long)a.vcap;
     const unsigned long long b0 = s_blk.x;
-    const unsigned long long n0 = b0 < vc ? min((unsigned long long)s_blk.y, vc - b0) : 0ull;
+    const unsigned long long n0 = b0 < vc ? min((unsigned long long)blk_candidates(s_blk.y), vc - b0) : 0ull;
     float pose[6] = {0, 0, 0, 0, 0, 0};
     for (unsigned long long u = threadIdx.x; u < n0; u += kProjBwdThreads) {
         const uint32_t sl = (uint32_t)(b0 + u);

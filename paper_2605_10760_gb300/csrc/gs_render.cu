@@ -124,24 +124,6 @@ __device__ __forceinline__ uint32_t warp_region_mask(const float4 &r0, const flo
 
 constexpr unsigned long long kTmaWaitLimit = 1ull << 22;   // polls of a batch's mbarrier before giving up
 
-// Claim order: the binning lists every (view, tile) item under its claim class (class 0 the
-// longest lists); coff[k] is the number of items in classes below k (coff[kClaimClasses] = all),
-// so the counter's value c falls in the class k with coff[k] <= c < coff[k + 1].
-__device__ __forceinline__ void claim_offsets(const DevStatus *st, uint32_t *coff) {
-    if (threadIdx.x < 32) {
-        static_assert(kClaimClasses == 32, "one class per lane");
-        const uint32_t x = st->claim_cnt[threadIdx.x];
-        uint32_t y = x;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t t = __shfl_up_sync(0xffffffffu, y, o);
-            if ((int)threadIdx.x >= o) y += t;
-        }
-        coff[threadIdx.x] = y - x;
-        if (threadIdx.x == 31) coff[32] = y;
-    }
-}
-
 // Next work item of a persistent compositing CTA (thread 0), -1 when all are taken.  Every CTA
 // makes exactly one claim past the last item; the CTA that draws the last of those (every other
 // claim of the launch is made by then) returns the counter to zero for the next launch.  Class
@@ -155,17 +137,12 @@ __device__ __forceinline__ long long claim_item(DevStatus *st, uint32_t *ctr, co
         if (c == total + (long long)gridDim.x - 1) *ctr = 0u;
         return -1;
     }
-    int k = 0;   // the largest k with coff[k] <= c (coff[0] = 0)
-#pragma unroll
-    for (int step = kClaimClasses / 2; step > 0; step >>= 1)
-        if ((long long)coff[k + step] <= c) k += step;
-    const long long r = c - (long long)coff[k];
-    const uint32_t g = r < G ? clist[(size_t)k * G + r] : 0xffffffffu;
-    if ((long long)g >= G) {
+    const long long g = claim_at(coff, clist, G, c);
+    if (g >= G) {
         record_error(st, GS_ERR_DEVICE_FAULT, 10);
         return c;
     }
-    return (long long)g;
+    return g;
 }
 
 // A CTA leaving early (after a failed wait, an error already recorded) claims until it draws a
