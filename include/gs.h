@@ -95,8 +95,9 @@ typedef struct gs_params {
     float bg[3];
     int32_t sort_mode;                 /* GS_SORT_ONESWEEP or GS_SORT_TILE_BUCKET */
     int32_t batch_records;             /* list entries staged per TMA batch by the compositing kernels:
-                                          0 = min(256, tile pixels); else 64, 128 or 256, at most the
-                                          tile's pixel count (a tuning knob: results do not change) */
+                                          0 = chosen by the library (128 or min(256, tile pixels)); else
+                                          64, 128 or 256, at most the tile's pixel count (a tuning knob:
+                                          results do not change) */
 } gs_params;
 
 /* One rendering problem: V views of one or more scenes (agents' submaps) whose Gaussians are

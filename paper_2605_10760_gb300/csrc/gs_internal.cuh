@@ -311,6 +311,29 @@ __device__ __forceinline__ float2 spec_expf2(float2 x) {
     return e;
 }
 
+// spec_expf2(-s) for components s in [0, 80], bit for bit.  Everything runs on s and -r with the signs of
+// the odd coefficients turned (rounding to nearest is symmetric), so nothing is negated; no range is
+// clamped; and since the result stays normal, its multiplication by 2^k is an addition to the exponent
+// field (t's low bits hold k, and 0x4B400000 << 23 vanishes).  Other components give garbage.
+__device__ __forceinline__ float2 spec_exp_neg(float2 s) {
+    using fp2::splat;
+    const float kShift = 12582912.0f;
+    const float2 t = fp2::add(fp2::mul(s, splat(-0x1.715476p+0f)), splat(kShift));
+    const float2 kf = fp2::add(t, splat(-kShift));
+    float2 r = fp2::fma(kf, splat(0x1.62e4p-1f), s);         // -r of spec_expf
+    r = fp2::fma(kf, splat(0x1.7f7d1cp-20f), r);
+    float2 p = fp2::fma(splat(-0x1.a01a02p-13f), r, splat(0x1.6c16c2p-10f));
+    p = fp2::fma(p, r, splat(-0x1.111112p-7f));
+    p = fp2::fma(p, r, splat(0x1.555556p-5f));
+    p = fp2::fma(p, r, splat(-0x1.555556p-3f));
+    p = fp2::fma(p, r, splat(0.5f));
+    p = fp2::fma(p, r, splat(-1.0f));
+    p = fp2::fma(p, r, splat(1.0f));
+    return make_float2(__uint_as_float((__float_as_uint(t.x) << 23) + __float_as_uint(p.x)),
+                       __uint_as_float((__float_as_uint(t.y) << 23) + __float_as_uint(p.y)));
+}
+constexpr float kFastCut = 80.0f;   // sigma cut-offs below it keep spec_exp_neg in range
+
 // spec_sigma at two pixels of one column (dy per pixel)
 __device__ __forceinline__ float2 spec_sigma2(float A, float B, float C, float dx, float2 dy) {
     const float2 q = fp2::fma(fp2::splat(fp::mul(A, dx)), fp2::splat(dx), fp2::mul(fp2::mul(fp2::splat(C), dy), dy));
