@@ -344,7 +344,7 @@ int gs_loss_l1_ssim(int32_t views, int32_t width, int32_t height, const float *r
  *    call clears what must start at zero itself.  Calls whose executions overlap on the GPU (on
  *    different streams, or from different host threads) race on the area and give wrong results:
  *    order them on one stream or synchronise between them.
- * The image planes are processed one after another, so it launches 2 kernels per plane plus 2. */
+ * The image planes are processed one after another, so it launches 2 kernels per plane plus 1. */
 #define GS_SSIM_NOALLOC_MAX_PLANE (1 << 20)
 int gs_loss_l1_ssim_noalloc(int32_t views, int32_t width, int32_t height, const float *rgb, const float *rgb_t,
                             float w_l1, float w_ssim, float *d_rgb, double *loss, void *stream);

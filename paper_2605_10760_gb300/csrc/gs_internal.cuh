@@ -311,6 +311,13 @@ __device__ __forceinline__ float2 spec_expf2(float2 x) {
     return e;
 }
 
+// s + x, exactly up to the rounding of the second float: the two-sum of s.x and x
+__device__ __forceinline__ void add_to_pair(float2 &s, float x) {
+    const float t = fp::add(s.x, x), b = fp::sub(t, s.x);
+    s.y = fp::add(s.y, fp::add(fp::sub(s.x, fp::sub(t, b)), fp::sub(x, b)));
+    s.x = t;
+}
+
 // spec_expf2(-s) for components s in [0, 80], bit for bit.  Everything runs on s and -r with the signs of
 // the odd coefficients turned (rounding to nearest is symmetric), so nothing is negated; no range is
 // clamped; and since the result stays normal, its multiplication by 2^k is an addition to the exponent

@@ -3,7 +3,7 @@
 // L1 (Eq. 4's photometric and depth terms): one pass per pixel producing the loss and its
 // gradient.  SSIM (Eq. 23's structural term): two tiled passes with an 11-tap separable Gaussian
 // (sigma 1.5, zero padding) in shared memory:
-//   pass 1 blurs x, y, x^2, y^2, xy and writes the per-pixel derivatives of the SSIM map with
+//   pass 1 blurs x, y, x^2, y^2, xy, sums the SSIM map and |x - y|, and writes the per-pixel derivatives of the SSIM map with
 //          respect to mu_x, E[x^2] and E[xy];
 //   pass 2 blurs those three maps (the adjoint of a zero-padded symmetric blur is the same blur)
 //          and combines dSSIM/dx = blur(dS/dmu_x) + 2 x blur(dS/dE[x^2]) + y blur(dS/dE[xy]),
@@ -134,165 +134,329 @@ static SsimTaps make_taps() {
     return t;
 }
 
-// Both passes map the 256 threads of a CTA as 32 columns x 8 rows: loads and the horizontal
-// filter walk rows ty, ty + 8, ... of column tx; the vertical filter gives each thread kVRows
-// consecutive output rows of its column and slides over the kVRows + 10 filtered rows they need,
-// so every filtered value is read from shared memory once per thread instead of once per tap.
-constexpr int kVRows = kSB / 8;
+// Both passes: 256 threads per 32 x 32 output tile.  The inputs are fetched 16 bytes at a time where the
+// planes allow it: 42 rows of 48 columns, from 8 left of the tile, so that every group of four is in or out as
+// a whole.  The horizontal filter gives a thread four adjacent columns of one row, so it loads 16 inputs for
+// four outputs; the vertical filter four rows of one column.  Values that take the same taps are the two
+// components of packed FP32x2 arithmetic: pass 1 filters (x, y) and (x^2, y^2) packed and x y alone, pass 2
+// (dS/dmu_x, dS/dE[x^2]) packed and dS/dE[xy] alone.  (The SSIM map's mean enters an FP64 loss and its bias
+// comes from the rounding of these sums, so their operations are part of the result: taps in ascending order,
+// w x rounded before it is added or meets its second factor.)  The pitches below and the order of the lanes in
+// the horizontal filter (hlane) keep every 16-byte shared access of eight lanes on 32 different banks.
+// 8 views of 1200 x 680 (19.6 M samples): pass 1 213 us (70 % of the issue slots; 392 MB take 58 us), pass 2
+// 173 us (63 %; 470 MB, 69 us); with one sample per load and scalar arithmetic 318 us and 279 us, plus 47 us
+// for a pass of its own for |x - y|.  The scalar
+// loads of other widths or alignments cost the 42 x 42 tile 7 guarded loads a thread instead of 2.
+constexpr int kSVR = 4;            // rows per thread in the vertical filter, columns in the horizontal one
+constexpr int kSC = 48;            // input columns, the tile's own from kSL
+constexpr int kSL = 8;
+constexpr int kHItems = (kSI + 3) / 4 * 32;   // (row, column group) pairs of the horizontal filter, padded
 
-struct Ssim1Smem {
-    float sx[kSI][kSI], sy[kSI][kSI];
-    float h[5][kSI][kSB];
+struct __align__(16) Ssim1Smem {
+    float2 xy[kSI][kSC + 2];
+    float4 h[kSI][kSB + 4];        // filtered x, y, x^2, y^2 of column c at c ^ (c >> 2)
+    float hxy[kSI][kSB + 8];       // filtered x y, likewise
 };
-struct Ssim2Smem {
-    float s[3][kSI][kSI];
-    float h[3][kSI][kSB];
+struct __align__(16) Ssim2Smem {
+    float2 a[kSI][kSC + 2];        // dS/dmu_x, dS/dE[x^2]
+    float b[kSI][kSC];             // dS/dE[xy]
+    float2 ha[kSI][kSB + 2];
+    float hb[kSI][kSB + 16];
 };
 
-template <int M>
-__device__ __forceinline__ void ssim_vpass(const float (&h)[M][kSI][kSB], const SsimTaps &tp, int tx, int ty,
-                                           float (&out)[M][kVRows]) {
+// item i of the horizontal filter: four lanes along a row, the next four on the row below it
+__device__ __forceinline__ int hlane_row(int i) { return (i >> 5) * 4 + ((i >> 2) & 1) + ((i >> 3) & 2); }
+__device__ __forceinline__ int hlane_group(int i) { return (i & 3) + ((i >> 1) & 4); }
+
+// p[0..3] of a row whose columns gx..gx+3 may lie outside [0, W) (all or none of them with VEC)
+template <bool VEC>
+__device__ __forceinline__ float4 load4(const float *row, int gx, int W) {
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (VEC) {
+        if (gx >= 0 && gx < W) v = *reinterpret_cast<const float4 *>(row + gx);
+    } else {
+        if (gx >= 0 && gx < W) v.x = row[gx];
+        if (gx + 1 >= 0 && gx + 1 < W) v.y = row[gx + 1];
+        if (gx + 2 >= 0 && gx + 2 < W) v.z = row[gx + 2];
+        if (gx + 3 >= 0 && gx + 3 < W) v.w = row[gx + 3];
+    }
+    return v;
+}
+
+// (a, b) summed over the CTA (256 threads) and added to *pa, *pb: as float pairs within a warp, in FP64
+// across warps
+__device__ __forceinline__ void block_add2(float2 a, float2 b, double *pa, double *pb) {
+    __shared__ double2 s_part[8];
 #pragma unroll
-    for (int m = 0; m < M; ++m)
+    for (int o = 16; o > 0; o >>= 1) {
+        const float ax = __shfl_xor_sync(0xffffffffu, a.x, o), ay = __shfl_xor_sync(0xffffffffu, a.y, o);
+        const float bx = __shfl_xor_sync(0xffffffffu, b.x, o), by = __shfl_xor_sync(0xffffffffu, b.y, o);
+        a.y = fp::add(a.y, ay);
+        b.y = fp::add(b.y, by);
+        add_to_pair(a, ax);
+        add_to_pair(b, bx);
+    }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (lane == 0) s_part[warp] = make_double2((double)a.x + a.y, (double)b.x + b.y);
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        double v = 0.0;
+        for (int w = 0; w < 8; ++w) v += threadIdx.x ? s_part[w].y : s_part[w].x;
+        if (v != 0.0) atomicAdd(threadIdx.x ? pb : pa, v);
+    }
+}
+
+// Pass 1 of one tile of one plane: x, y (x optionally as fl(fl(ea x) + eb)), zero padding; the blurred
+// moments, the SSIM map and |x - y| summed over the thread's share, and the three per-pixel derivatives
+// dS/dmu_x, dS/dE[x^2], dS/dE[xy] (scaled by inv_n) written for pass 2.
+template <bool EXPO, bool VEC>
+__device__ __forceinline__ void ssim_pass1_tile(Ssim1Smem &sm, int W, int H, const float *xp, const float *yp, float ea,
+                                                float eb, const SsimTaps &tp, float inv_n, float *dmu, float *dexx,
+                                                float *dexy, float2 &s_ssim, float2 &s_l1) {
+    const int x0 = blockIdx.x * kSB - kSL, y0 = blockIdx.y * kSB - kR;
+    s_ssim = s_l1 = make_float2(0.f, 0.f);
+    float4 xv[2], yv[2];
 #pragma unroll
-        for (int q = 0; q < kVRows; ++q) out[m][q] = 0.f;
+    for (int part = 0; part < 2; ++part) {   // every load before the first store
+        const int i = threadIdx.x + 256 * part, r = i / (kSC / 4), c = (i - r * (kSC / 4)) * 4;
+        const int gx = x0 + c, gy = y0 + r;
+        xv[part] = yv[part] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r < kSI && gy >= 0 && gy < H) {
+            xv[part] = load4<VEC>(xp + (long long)gy * W, gx, W);
+            yv[part] = load4<VEC>(yp + (long long)gy * W, gx, W);
+            if (EXPO) {   // the padding stays zero
+                float4 &x = xv[part];
+                if (gx >= 0 && gx < W) x.x = fp::add(fp::mul(ea, x.x), eb);
+                if (VEC ? gx >= 0 && gx < W : gx + 1 >= 0 && gx + 1 < W) x.y = fp::add(fp::mul(ea, x.y), eb);
+                if (VEC ? gx >= 0 && gx < W : gx + 2 >= 0 && gx + 2 < W) x.z = fp::add(fp::mul(ea, x.z), eb);
+                if (VEC ? gx >= 0 && gx < W : gx + 3 >= 0 && gx + 3 < W) x.w = fp::add(fp::mul(ea, x.w), eb);
+            }
+        }
+    }
 #pragma unroll
-    for (int j = 0; j < kVRows + 2 * kR; ++j) {
-        float hv[M];
+    for (int part = 0; part < 2; ++part) {
+        const int i = threadIdx.x + 256 * part, r = i / (kSC / 4), c = (i - r * (kSC / 4)) * 4;
+        if (r >= kSI) break;
+        float4 *d = reinterpret_cast<float4 *>(&sm.xy[r][c]);
+        d[0] = make_float4(xv[part].x, yv[part].x, xv[part].y, yv[part].y);
+        d[1] = make_float4(xv[part].z, yv[part].z, xv[part].w, yv[part].w);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < kHItems; i += 256) {
+        const int r = hlane_row(i), t = hlane_group(i);
+        if (r >= kSI) continue;
+        float2 m[kSVR], q[kSVR];
+        float p[kSVR];
 #pragma unroll
-        for (int m = 0; m < M; ++m) hv[m] = h[m][ty * kVRows + j][tx];
+        for (int j = 0; j < kSVR; ++j) {
+            m[j] = q[j] = make_float2(0.f, 0.f);
+            p[j] = 0.f;
+        }
+        // output column 4 t + j takes inputs 4 t + j + kSL - kR + (0 .. 2 kR)
+        const float4 *src = reinterpret_cast<const float4 *>(&sm.xy[r][4 * t]);
+        constexpr int kFirst = kSL - kR;
 #pragma unroll
-        for (int q = 0; q < kVRows; ++q) {
-            const int k = j - q;
-            if (k >= 0 && k <= 2 * kR) {
+        for (int u = kFirst / 2; u <= (kFirst + kSVR - 1 + 2 * kR) / 2; ++u) {
+            const float4 f = src[u];
 #pragma unroll
-                for (int m = 0; m < M; ++m) out[m][q] += tp.w[k] * hv[m];
+            for (int e = 0; e < 2; ++e) {
+                const int k = 2 * u + e - kFirst;
+                const float2 v = e ? make_float2(f.z, f.w) : make_float2(f.x, f.y);
+#pragma unroll
+                for (int j = 0; j < kSVR; ++j) {
+                    if (k - j >= 0 && k - j <= 2 * kR) {
+                        const float2 wv = fp2::mul(fp2::splat(tp.w[k - j]), v);
+                        m[j] = fp2::add(wv, m[j]);
+                        q[j] = fp2::fma(wv, v, q[j]);
+                        p[j] = fmaf(wv.x, v.y, p[j]);
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < kSVR; ++j) {
+            const int c = (4 * t + j) ^ t;
+            sm.h[r][c] = make_float4(m[j].x, m[j].y, q[j].x, q[j].y);
+            sm.hxy[r][c] = p[j];
+        }
+    }
+    __syncthreads();
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, tc = tx ^ (tx >> 2);
+    float2 m[kSVR], q[kSVR];
+    float p[kSVR];
+#pragma unroll
+    for (int j = 0; j < kSVR; ++j) {
+        m[j] = q[j] = make_float2(0.f, 0.f);
+        p[j] = 0.f;
+    }
+#pragma unroll
+    for (int k = 0; k < kSVR + 2 * kR; ++k) {
+        const float4 v = sm.h[ty * kSVR + k][tc];
+        const float vp = sm.hxy[ty * kSVR + k][tc];
+#pragma unroll
+        for (int j = 0; j < kSVR; ++j) {
+            if (k - j >= 0 && k - j <= 2 * kR) {
+                const float2 w = fp2::splat(tp.w[k - j]);
+                m[j] = fp2::fma(w, make_float2(v.x, v.y), m[j]);
+                q[j] = fp2::fma(w, make_float2(v.z, v.w), q[j]);
+                p[j] = fmaf(tp.w[k - j], vp, p[j]);
+            }
+        }
+    }
+    const int gx = blockIdx.x * kSB + tx, gy0 = blockIdx.y * kSB + ty * kSVR;
+    if (gx >= W) return;
+#pragma unroll
+    for (int j = 0; j < kSVR; ++j) {
+        if (gy0 + j >= H) break;
+        const float mx = m[j].x, my = m[j].y, exx = q[j].x, eyy = q[j].y, exy = p[j];
+        const float vx = exx - mx * mx, vy = eyy - my * my, cxy = exy - mx * my;
+        const float A1 = 2.f * mx * my + kC1, A2 = 2.f * cxy + kC2;
+        const float B1 = mx * mx + my * my + kC1, B2 = vx + vy + kC2;
+        const float iB = 1.f / (B1 * B2), iB1 = iB * B2, iB2 = iB * B1;
+        const float S = A1 * A2 * iB;
+        const float2 v = sm.xy[ty * kSVR + j + kR][tx + kSL];
+        add_to_pair(s_ssim, S);
+        add_to_pair(s_l1, fabsf(v.x - v.y));
+        const long long o = (long long)(gy0 + j) * W + gx;
+        dmu[o] = inv_n * ((2.f * my * A2 - 2.f * my * A1) * iB - S * (2.f * mx * iB1 - 2.f * mx * iB2));
+        dexx[o] = inv_n * (-S * iB2);
+        dexy[o] = inv_n * (2.f * A1 * iB);
+    }
+}
+
+// Pass 2 of one tile: the three derivative maps blurred (the adjoint of a zero-padded symmetric
+// blur is the same blur); ga = (blur(dS/dmu_x), blur(dS/dE[x^2])), gb = blur(dS/dE[xy]) for the thread's
+// kSVR outputs.
+template <bool VEC>
+__device__ __forceinline__ void ssim_pass2_tile(Ssim2Smem &sm, int W, int H, const float *dmu, const float *dexx,
+                                                const float *dexy, const SsimTaps &tp, float2 (&ga)[kSVR],
+                                                float (&gb)[kSVR]) {
+    const int x0 = blockIdx.x * kSB - kSL, y0 = blockIdx.y * kSB - kR;
+    float4 v0[2], v1[2], v2[2];
+#pragma unroll
+    for (int part = 0; part < 2; ++part) {
+        const int i = threadIdx.x + 256 * part, r = i / (kSC / 4), c = (i - r * (kSC / 4)) * 4;
+        const int gx = x0 + c, gy = y0 + r;
+        v0[part] = v1[part] = v2[part] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r < kSI && gy >= 0 && gy < H) {
+            const long long o = (long long)gy * W;
+            v0[part] = load4<VEC>(dmu + o, gx, W);
+            v1[part] = load4<VEC>(dexx + o, gx, W);
+            v2[part] = load4<VEC>(dexy + o, gx, W);
+        }
+    }
+#pragma unroll
+    for (int part = 0; part < 2; ++part) {
+        const int i = threadIdx.x + 256 * part, r = i / (kSC / 4), c = (i - r * (kSC / 4)) * 4;
+        if (r >= kSI) break;
+        float4 *d = reinterpret_cast<float4 *>(&sm.a[r][c]);
+        d[0] = make_float4(v0[part].x, v1[part].x, v0[part].y, v1[part].y);
+        d[1] = make_float4(v0[part].z, v1[part].z, v0[part].w, v1[part].w);
+        *reinterpret_cast<float4 *>(&sm.b[r][c]) = v2[part];
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < kHItems; i += 256) {
+        const int r = hlane_row(i), t = hlane_group(i);
+        if (r >= kSI) continue;
+        float2 a[kSVR];
+        float b[kSVR];
+#pragma unroll
+        for (int j = 0; j < kSVR; ++j) {
+            a[j] = make_float2(0.f, 0.f);
+            b[j] = 0.f;
+        }
+        const float4 *sa = reinterpret_cast<const float4 *>(&sm.a[r][4 * t]);
+        const float4 *sb = reinterpret_cast<const float4 *>(&sm.b[r][4 * t]);
+        constexpr int kFirst = kSL - kR;
+#pragma unroll
+        for (int u = 0; u <= (kFirst + kSVR - 1 + 2 * kR) / 4; ++u) {
+            const float4 f0 = sa[2 * u], f1 = sa[2 * u + 1], fb = sb[u];
+            const float2 va[4] = {make_float2(f0.x, f0.y), make_float2(f0.z, f0.w), make_float2(f1.x, f1.y),
+                                  make_float2(f1.z, f1.w)};
+            const float vb[4] = {fb.x, fb.y, fb.z, fb.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int k = 4 * u + e - kFirst;
+#pragma unroll
+                for (int j = 0; j < kSVR; ++j) {
+                    if (k - j >= 0 && k - j <= 2 * kR) {
+                        a[j] = fp2::fma(fp2::splat(tp.w[k - j]), va[e], a[j]);
+                        b[j] = fmaf(tp.w[k - j], vb[e], b[j]);
+                    }
+                }
+            }
+        }
+        float4 *da = reinterpret_cast<float4 *>(&sm.ha[r][4 * t]);
+        da[0] = make_float4(a[0].x, a[0].y, a[1].x, a[1].y);
+        da[1] = make_float4(a[2].x, a[2].y, a[3].x, a[3].y);
+        *reinterpret_cast<float4 *>(&sm.hb[r][4 * t]) = make_float4(b[0], b[1], b[2], b[3]);
+    }
+    __syncthreads();
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+#pragma unroll
+    for (int j = 0; j < kSVR; ++j) {
+        ga[j] = make_float2(0.f, 0.f);
+        gb[j] = 0.f;
+    }
+#pragma unroll
+    for (int k = 0; k < kSVR + 2 * kR; ++k) {
+        const float2 va = sm.ha[ty * kSVR + k][tx];
+        const float vb = sm.hb[ty * kSVR + k][tx];
+#pragma unroll
+        for (int j = 0; j < kSVR; ++j) {
+            if (k - j >= 0 && k - j <= 2 * kR) {
+                ga[j] = fp2::fma(fp2::splat(tp.w[k - j]), va, ga[j]);
+                gb[j] = fmaf(tp.w[k - j], vb, gb[j]);
             }
         }
     }
 }
 
-// Pass 1 of one tile of one plane: x, y (x optionally as fl(fl(ea x) + eb)), zero padding; the
-// five blurred moments, the SSIM map summed into the return value and the three per-pixel
-// derivatives dS/dmu_x, dS/dE[x^2], dS/dE[xy] (scaled by inv_n) written for pass 2.
-__device__ __forceinline__ double ssim_pass1_tile(Ssim1Smem &sm, int W, int H, const float *xp, const float *yp,
-                                                  bool expo, float ea, float eb, const SsimTaps &tp, float inv_n,
-                                                  float *dmu, float *dexx, float *dexy) {
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int x0 = blockIdx.x * kSB - kR, y0 = blockIdx.y * kSB - kR;
-    for (int r = ty; r < kSI; r += 8)
-        for (int c = tx; c < kSI; c += 32) {
-            const int gx = x0 + c, gy = y0 + r;
-            const bool in = gx >= 0 && gx < W && gy >= 0 && gy < H;
-            const long long o = (long long)gy * W + gx;
-            const float xv = in ? xp[o] : 0.f;
-            sm.sx[r][c] = in ? (expo ? fp::add(fp::mul(ea, xv), eb) : xv) : 0.f;   // zero padding
-            sm.sy[r][c] = in ? yp[o] : 0.f;
-        }
-    __syncthreads();
-    for (int r = ty; r < kSI; r += 8) {
-        float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f, a4 = 0.f;
+// the images at a thread's outputs, asked for before pass 2 waits for its tile (8 views of 1200 x 680: 235 us
+// with these loads after the filter, 173 us before it)
+__device__ __forceinline__ void load_outputs(const float *x, const float *y, int W, int H, int gx, int gy0,
+                                             float (&px)[kSVR], float (&py)[kSVR]) {
 #pragma unroll
-        for (int k = 0; k <= 2 * kR; ++k) {
-            const float xv = sm.sx[r][tx + k], yv = sm.sy[r][tx + k], w = tp.w[k];
-            a0 += w * xv;
-            a1 += w * yv;
-            a2 += w * xv * xv;
-            a3 += w * yv * yv;
-            a4 += w * xv * yv;
-        }
-        sm.h[0][r][tx] = a0; sm.h[1][r][tx] = a1; sm.h[2][r][tx] = a2; sm.h[3][r][tx] = a3; sm.h[4][r][tx] = a4;
+    for (int j = 0; j < kSVR; ++j) {
+        const bool in = gx < W && gy0 + j < H;
+        const long long o = (long long)(gy0 + j) * W + gx;
+        px[j] = in ? x[o] : 0.f;
+        py[j] = in ? y[o] : 0.f;
     }
-    __syncthreads();
-    float v5[5][kVRows];
-    ssim_vpass<5>(sm.h, tp, tx, ty, v5);
-    double acc = 0.0;
-#pragma unroll
-    for (int q = 0; q < kVRows; ++q) {
-        const int gx = blockIdx.x * kSB + tx, gy = blockIdx.y * kSB + ty * kVRows + q;
-        if (gx >= W || gy >= H) continue;
-        const float mx = v5[0][q], my = v5[1][q], exx = v5[2][q], eyy = v5[3][q], exy = v5[4][q];
-        const float vx = exx - mx * mx, vy = eyy - my * my, cxy = exy - mx * my;
-        const float A1 = 2.f * mx * my + kC1, A2 = 2.f * cxy + kC2;
-        const float B1 = mx * mx + my * my + kC1, B2 = vx + vy + kC2;
-        const float iB = 1.f / (B1 * B2);
-        const float S = A1 * A2 * iB;
-        acc += (double)S;
-        const long long o = (long long)gy * W + gx;
-        dmu[o] = inv_n * ((2.f * my * A2 - 2.f * my * A1) * iB - S * (2.f * mx / B1 - 2.f * mx / B2));
-        dexx[o] = inv_n * (-S / B2);
-        dexy[o] = inv_n * (2.f * A1 * iB);
-    }
-    return acc;
 }
 
-// Pass 2 of one tile: the three derivative maps blurred (the adjoint of a zero-padded symmetric
-// blur is the same blur); out[0..2] = blur(dS/dmu_x), blur(dS/dE[x^2]), blur(dS/dE[xy]) for the
-// thread's kVRows outputs.
-__device__ __forceinline__ void ssim_pass2_tile(Ssim2Smem &sm, int W, int H, const float *dmu, const float *dexx,
-                                                const float *dexy, const SsimTaps &tp, float (&out)[3][kVRows]) {
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int x0 = blockIdx.x * kSB - kR, y0 = blockIdx.y * kSB - kR;
-    for (int r = ty; r < kSI; r += 8)
-        for (int c = tx; c < kSI; c += 32) {
-            const int gx = x0 + c, gy = y0 + r;
-            const bool in = gx >= 0 && gx < W && gy >= 0 && gy < H;
-            const long long o = (long long)gy * W + gx;
-            sm.s[0][r][c] = in ? dmu[o] : 0.f;
-            sm.s[1][r][c] = in ? dexx[o] : 0.f;
-            sm.s[2][r][c] = in ? dexy[o] : 0.f;
-        }
-    __syncthreads();
-    for (int r = ty; r < kSI; r += 8) {
-        float a0 = 0.f, a1 = 0.f, a2 = 0.f;
-#pragma unroll
-        for (int k = 0; k <= 2 * kR; ++k) {
-            const float w = tp.w[k];
-            a0 += w * sm.s[0][r][tx + k];
-            a1 += w * sm.s[1][r][tx + k];
-            a2 += w * sm.s[2][r][tx + k];
-        }
-        sm.h[0][r][tx] = a0; sm.h[1][r][tx] = a1; sm.h[2][r][tx] = a2;
-    }
-    __syncthreads();
-    ssim_vpass<3>(sm.h, tp, tx, ty, out);
-}
-
-// pass 1: per image plane (view * 3 + channel) = blockIdx.z, tile (bx, by)
-__global__ void __launch_bounds__(256) k_ssim1(int W, int H, const float *x, const float *y, SsimTaps tp,
-                                               float inv_n, float *dmu, float *dexx, float *dexy, double *ssim_sum) {
+// pass 1: per image plane (view * 3 + channel) = blockIdx.z, tile (bx, by); sums[0] += |x - y|, sums[1] += SSIM
+template <bool VEC>
+__global__ void __launch_bounds__(256, 4) k_ssim1(int W, int H, const float *x, const float *y, SsimTaps tp,
+                                                  float inv_n, float *dmu, float *dexx, float *dexy, double *sums) {
     __shared__ Ssim1Smem sm;
     const long long off = (long long)blockIdx.z * W * H;
-    const double acc = ssim_pass1_tile(sm, W, H, x + off, y + off, false, 1.f, 0.f, tp, inv_n, dmu + off, dexx + off,
-                                       dexy + off);
-    block_add_double(acc, ssim_sum);
+    float2 s, l;
+    ssim_pass1_tile<false, VEC>(sm, W, H, x + off, y + off, 1.f, 0.f, tp, inv_n, dmu + off, dexx + off, dexy + off, s, l);
+    block_add2(l, s, sums, sums + 1);
 }
 
 // pass 2: blur the three derivative maps and combine with the L1 gradient
-__global__ void __launch_bounds__(256) k_ssim2(int W, int H, const float *x, const float *y, SsimTaps tp,
-                                               const float *dmu, const float *dexx, const float *dexy, float l1_scale,
-                                               float w_ssim, float *d_rgb) {
+template <bool VEC>
+__global__ void __launch_bounds__(256, 4) k_ssim2(int W, int H, const float *x, const float *y, SsimTaps tp,
+                                                  const float *dmu, const float *dexx, const float *dexy, float l1_scale,
+                                                  float w_ssim, float *d_rgb) {
     __shared__ Ssim2Smem sm;
     const long long off = (long long)blockIdx.z * W * H;
-    float b[3][kVRows];
-    ssim_pass2_tile(sm, W, H, dmu + off, dexx + off, dexy + off, tp, b);
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int gx = blockIdx.x * kSB + (threadIdx.x & 31), gy0 = blockIdx.y * kSB + (threadIdx.x >> 5) * kSVR;
+    float2 ga[kSVR];
+    float gb[kSVR], px[kSVR], py[kSVR];
+    load_outputs(x + off, y + off, W, H, gx, gy0, px, py);
+    ssim_pass2_tile<VEC>(sm, W, H, dmu + off, dexx + off, dexy + off, tp, ga, gb);
+    if (gx >= W) return;
 #pragma unroll
-    for (int q = 0; q < kVRows; ++q) {
-        const int gx = blockIdx.x * kSB + tx, gy = blockIdx.y * kSB + ty * kVRows + q;
-        if (gx >= W || gy >= H) continue;
-        const long long o = off + (long long)gy * W + gx;
-        const float xv = x[o], yv = y[o];
-        const float gs = b[0][q] + 2.f * xv * b[1][q] + yv * b[2][q];
+    for (int j = 0; j < kSVR; ++j) {
+        if (gy0 + j >= H) break;
+        const long long o = off + (long long)(gy0 + j) * W + gx;
+        const float xv = px[j], yv = py[j];
+        const float gs = ga[j].x + 2.f * xv * ga[j].y + yv * gb[j];
         d_rgb[o] = l1_scale * sgnf(xv - yv) - w_ssim * gs;
     }
-}
-
-__global__ void k_l1_sum(long long n, const float *x, const float *y, double *out) {
-    double acc = 0.0;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        acc += (double)fabsf(x[i] - y[i]);
-    block_add_double(acc, out);
 }
 
 __global__ void k_ssim_finish(double *scratch_sums, float w_l1, float w_ssim, double inv_n, double *loss) {
@@ -300,8 +464,26 @@ __global__ void k_ssim_finish(double *scratch_sums, float w_l1, float w_ssim, do
     *loss = w_l1 * scratch_sums[0] * inv_n + w_ssim * (1.0 - scratch_sums[1] * inv_n);
 }
 
+// 16-byte accesses: every row of every plane starts on such a boundary
+static bool ssim_vec(int W, const float *x, const float *y, const float *maps) {
+    return W % 4 == 0 && aligned16(x) && aligned16(y) && aligned16(maps);
+}
+
 size_t ssim_scratch_bytes(int V, int W, int H) {
     return 256 + 3 * sizeof(float) * (size_t)V * 3 * W * H;
+}
+
+// both passes over grid.z planes
+static void launch_ssim(dim3 grid, int W, int H, const float *x, const float *y, const SsimTaps &taps, float inv_n,
+                        float *dmu, float *dexx, float *dexy, double *sums, float l1_scale, float w_ssim, float *d_rgb,
+                        cudaStream_t s) {
+    if (ssim_vec(W, x, y, dmu)) {
+        k_ssim1<true><<<grid, 256, 0, s>>>(W, H, x, y, taps, inv_n, dmu, dexx, dexy, sums);
+        k_ssim2<true><<<grid, 256, 0, s>>>(W, H, x, y, taps, dmu, dexx, dexy, l1_scale, w_ssim, d_rgb);
+    } else {
+        k_ssim1<false><<<grid, 256, 0, s>>>(W, H, x, y, taps, inv_n, dmu, dexx, dexy, sums);
+        k_ssim2<false><<<grid, 256, 0, s>>>(W, H, x, y, taps, dmu, dexx, dexy, l1_scale, w_ssim, d_rgb);
+    }
 }
 
 int launch_loss_l1_ssim(int V, int W, int H, const float *rgb, const float *rgb_t, float w_l1, float w_ssim,
@@ -314,11 +496,9 @@ int launch_loss_l1_ssim(int V, int W, int H, const float *rgb, const float *rgb_
     if (cudaMemsetAsync(sums, 0, 2 * sizeof(double), s) != cudaSuccess) return GS_ERR_CUDA;
     dim3 grid((W + kSB - 1) / kSB, (H + kSB - 1) / kSB, 3 * V);
     const float inv_n = (float)(1.0 / (double)n);
-    k_l1_sum<<<device_sm_count() * 4, 256, 0, s>>>(n, rgb, rgb_t, sums);
-    k_ssim1<<<grid, 256, 0, s>>>(W, H, rgb, rgb_t, taps, inv_n, dmu, dexx, dexy, sums + 1);
-    k_ssim2<<<grid, 256, 0, s>>>(W, H, rgb, rgb_t, taps, dmu, dexx, dexy, w_l1 * inv_n, w_ssim, d_rgb);
+    launch_ssim(grid, W, H, rgb, rgb_t, taps, inv_n, dmu, dexx, dexy, sums, w_l1 * inv_n, w_ssim, d_rgb, s);
     k_ssim_finish<<<1, 1, 0, s>>>(sums, w_l1, w_ssim, 1.0 / (double)n, loss);
-    count_launches(4);
+    count_launches(3);
     return check_launch();
 }
 
@@ -368,16 +548,14 @@ int launch_loss_l1_ssim_noalloc(int V, int W, int H, const float *rgb, const flo
     float *dexx = dmu + plane, *dexy = dexx + plane;
     if (cudaMemsetAsync(sums, 0, 2 * sizeof(double), s) != cudaSuccess) return GS_ERR_CUDA;
     const float inv_n = (float)(1.0 / (double)n);
-    k_l1_sum<<<device_sm_count() * 4, 256, 0, s>>>(n, rgb, rgb_t, sums);
     dim3 grid((W + kSB - 1) / kSB, (H + kSB - 1) / kSB, 1);
     for (long long p = 0; p < 3LL * V; ++p) {
         const long long off = p * plane;
-        k_ssim1<<<grid, 256, 0, s>>>(W, H, rgb + off, rgb_t + off, taps, inv_n, dmu, dexx, dexy, sums + 1);
-        k_ssim2<<<grid, 256, 0, s>>>(W, H, rgb + off, rgb_t + off, taps, dmu, dexx, dexy, w_l1 * inv_n, w_ssim,
-                                     d_rgb + off);
+        launch_ssim(grid, W, H, rgb + off, rgb_t + off, taps, inv_n, dmu, dexx, dexy, sums, w_l1 * inv_n, w_ssim,
+                    d_rgb + off, s);
     }
     k_ssim_finish<<<1, 1, 0, s>>>(sums, w_l1, w_ssim, 1.0 / (double)n, loss);
-    count_launches((int)(2 + 6LL * V));
+    count_launches((int)(1 + 6LL * V));
     return check_launch();
 }
 
@@ -507,64 +685,59 @@ struct RefineArgs {
     float *dmu, *dexx, *dexy;
 };
 
-__global__ void k_refine_l1(RefineArgs a) {
-    const long long HWn = (long long)a.W * a.H, total = (long long)a.V * HWn;
-    float acc_rgb = 0.f, acc_d = 0.f;
+// the depth term
+__global__ void __launch_bounds__(256) k_refine_depth(RefineArgs a) {
+    const long long total = (long long)a.V * a.W * a.H;
+    float2 acc = make_float2(0.f, 0.f);
     const float sc_d = (float)((double)a.w_depth / (double)total);
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-        const long long v = i / HWn, p = i - v * HWn;
-        const float ea = spec_expf(a.expo[2 * v]), eb = a.expo[2 * v + 1];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const long long idx = (3 * v + c) * HWn + p;
-            acc_rgb += fabsf(fp::add(fp::mul(ea, a.rgb[idx]), eb) - a.rgb_t[idx]);
-        }
-        if (a.depth && a.d_depth) {
-            const float d = a.depth[i] - a.depth_t[i];
-            acc_d += fabsf(d);
-            a.d_depth[i] = sgnf(d) * sc_d;
-        }
+        const float d = a.depth[i] - a.depth_t[i];
+        add_to_pair(acc, fabsf(d));
+        a.d_depth[i] = sgnf(d) * sc_d;
     }
-    block_add_double((double)acc_rgb, a.sums);
-    block_add_double((double)acc_d, a.sums + 2);
+    block_add_double((double)acc.x + acc.y, a.sums + 2);
 }
 
-__global__ void __launch_bounds__(256) k_refine_ssim1(RefineArgs a, SsimTaps tp, float inv_n) {
+template <bool VEC>
+__global__ void __launch_bounds__(256, 4) k_refine_ssim1(RefineArgs a, SsimTaps tp, float inv_n) {
     __shared__ Ssim1Smem sm;
     const long long plane = blockIdx.z;
     const int v = (int)(plane / 3);
     const float ea = spec_expf(a.expo[2 * v]), eb = a.expo[2 * v + 1];
     const long long off = plane * (long long)a.W * a.H;
-    const double acc = ssim_pass1_tile(sm, a.W, a.H, a.rgb + off, a.rgb_t + off, true, ea, eb, tp, inv_n,
-                                       a.dmu + off, a.dexx + off, a.dexy + off);
-    block_add_double(acc, a.sums + 1);
+    float2 s, l;
+    ssim_pass1_tile<true, VEC>(sm, a.W, a.H, a.rgb + off, a.rgb_t + off, ea, eb, tp, inv_n, a.dmu + off, a.dexx + off,
+                          a.dexy + off, s, l);
+    block_add2(l, s, a.sums, a.sums + 1);
 }
 
-__global__ void __launch_bounds__(256) k_refine_ssim2(RefineArgs a, SsimTaps tp, float l1_scale) {
+template <bool VEC>
+__global__ void __launch_bounds__(256, 4) k_refine_ssim2(RefineArgs a, SsimTaps tp, float l1_scale) {
     __shared__ Ssim2Smem sm;
     const int W = a.W, H = a.H;
     const long long plane = blockIdx.z;
     const int v = (int)(plane / 3);
     const float ea = spec_expf(a.expo[2 * v]), eb = a.expo[2 * v + 1];
     const long long off = plane * (long long)W * H;
-    float b[3][kVRows];
-    ssim_pass2_tile(sm, W, H, a.dmu + off, a.dexx + off, a.dexy + off, tp, b);
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    float2 ba[kSVR];
+    float bb[kSVR];
+    const int gx = blockIdx.x * kSB + (threadIdx.x & 31), gy0 = blockIdx.y * kSB + (threadIdx.x >> 5) * kSVR;
+    float px[kSVR], py[kSVR];
+    load_outputs(a.rgb + off, a.rgb_t + off, W, H, gx, gy0, px, py);
+    ssim_pass2_tile<VEC>(sm, W, H, a.dmu + off, a.dexx + off, a.dexy + off, tp, ba, bb);
     float ga = 0.f, gb = 0.f;
 #pragma unroll
-    for (int q = 0; q < kVRows; ++q) {
-        const int gx = blockIdx.x * kSB + tx, gy = blockIdx.y * kSB + ty * kVRows + q;
-        if (gx >= W || gy >= H) continue;
-        const long long o = off + (long long)gy * W + gx;
-        const float xv = a.rgb[o], yv = a.rgb_t[o];
+    for (int j = 0; j < kSVR; ++j) {
+        if (gx >= W || gy0 + j >= H) continue;
+        const long long o = off + (long long)(gy0 + j) * W + gx;
+        const float xv = px[j], yv = py[j];
         const float xt = fp::add(fp::mul(ea, xv), eb);       // I~ exactly as the FP32 L1 sign decision takes it
-        const float g = l1_scale * sgnf(xt - yv) - a.w_ssim * (b[0][q] + 2.f * xt * b[1][q] + yv * b[2][q]);
+        const float g = l1_scale * sgnf(xt - yv) - a.w_ssim * (ba[j].x + 2.f * xt * ba[j].y + yv * bb[j]);
         a.d_rgb[o] = ea * g;                                 // dL/dI^ = e^a dL/dI~
         ga += g * ea * xv;
         gb += g;
     }
-    block_add_double((double)ga, a.sums + 3 + v);
-    block_add_double((double)gb, a.sums + 3 + a.V + v);
+    block_add2(make_float2(ga, 0.f), make_float2(gb, 0.f), a.sums + 3 + v, a.sums + 3 + a.V + v);
 }
 
 __global__ void k_refine_finish(RefineArgs a, double inv_n) {
@@ -604,12 +777,18 @@ int launch_loss_refine(int V, int W, int H, const float *rgb, const float *rgb_t
     const float inv_n = (float)(1.0 / (double)n);
     const long long total = (long long)V * plane;
     const int g1 = (int)std::max<long long>(1, std::min<long long>((total + 255) / 256, (long long)device_sm_count() * 8));
-    k_refine_l1<<<g1, 256, 0, s>>>(a);
+    const bool use_depth = a.depth && a.d_depth;
+    if (use_depth) k_refine_depth<<<g1, 256, 0, s>>>(a);
     dim3 grid((W + kSB - 1) / kSB, (H + kSB - 1) / kSB, 3 * V);
-    k_refine_ssim1<<<grid, 256, 0, s>>>(a, taps, inv_n);
-    k_refine_ssim2<<<grid, 256, 0, s>>>(a, taps, w_l1 * inv_n);
+    if (ssim_vec(W, rgb, rgb_t, a.dmu)) {
+        k_refine_ssim1<true><<<grid, 256, 0, s>>>(a, taps, inv_n);
+        k_refine_ssim2<true><<<grid, 256, 0, s>>>(a, taps, w_l1 * inv_n);
+    } else {
+        k_refine_ssim1<false><<<grid, 256, 0, s>>>(a, taps, inv_n);
+        k_refine_ssim2<false><<<grid, 256, 0, s>>>(a, taps, w_l1 * inv_n);
+    }
     k_refine_finish<<<1, ((V + 31) / 32) * 32, 0, s>>>(a, 1.0 / (double)n);
-    count_launches(4);
+    count_launches(3 + use_depth);
     return check_launch();
 }
 

@@ -258,13 +258,6 @@ __device__ __forceinline__ void drain_after_timeout(RenderSmem<NB> &sm, const ui
     __syncthreads();
 }
 
-// s + x, exactly up to the rounding of the second float: the two-sum of s.x and x
-__device__ __forceinline__ void add_to_pair(float2 &s, float x) {
-    const float t = fp::add(s.x, x), b = fp::sub(t, s.x);
-    s.y = fp::add(s.y, fp::add(fp::sub(s.x, fp::sub(t, b)), fp::sub(x, b)));
-    s.x = t;
-}
-
 // Resident CTAs per SM (32 warps of 64 registers when whole batches are staged, else 40 of 48): with short
 // lists the chain of claim, range, copy and masks of the next tile is hidden by more warps, with long
 // ones the walk itself runs faster with more registers.
