@@ -3,11 +3,13 @@
 //  * k_sim3: the Sim(3) correction C = (s, R, t) acting on Gaussians (Eq. 19): mu' = s R mu + t,
 //    rotation q' = q_R (x) q, log-scales + ln s; opacity and colour copied.
 //  * Voxel sets: open-addressing hash sets of 64-bit keys (voxel index kappa(x) = floor(x / v) per
-//    axis, 21 bits per axis with offset 2^20) with linear probing; insertion by compare-and-swap,
-//    membership by probing to the first empty slot.  Probing is bounded by the capacity; a full
-//    table records GS_ERR_CAPACITY in the set's status word instead of looping.
-//  * k_add_boxes (Eq. 20): every voxel of [kappa(mu - k s), kappa(mu + k s)].
-//  * k_add_rays (Eq. 21): one thread per (keyframe, strided pixel) walks the voxels crossed by the
+//    axis, 21 bits per axis with offset 2^20); insertion by compare-and-swap, membership by probing
+//    to the first empty slot.  Blocks of 4 x 2 x 2 voxels hash to lines of 16 slots, so neighbouring
+//    voxels meet in one line (VoxProbe).  Probing is bounded by the capacity; a full table records
+//    GS_ERR_CAPACITY in the set's status word instead of looping.
+//  * k_add_boxes (Eq. 20): every voxel of [kappa(mu - k s), kappa(mu + k s)]; a warp spreads the
+//    voxels of its 32 boxes over its lanes.
+//  * k_add_rays (Eq. 21): one thread per (keyframe, strided pixel), a warp per 8 x 4 of them, walks the voxels crossed by the
 //    segment from the camera centre to the back-projected depth point, t in [0, 1), with a 3-D
 //    digital differential analyser (ties between axes go to the lowest axis).
 //  * k_keep (Eq. 22): keep a borrowed Gaussian iff kappa(mu) is in neither set.
@@ -23,64 +25,100 @@ namespace gs {
 constexpr unsigned long long kEmptyKey = ~0ull;
 constexpr int kKeyBits = 21;
 constexpr long long kKeyOff = 1LL << 20;
+constexpr int kMaxRaySteps = 1 << 16;  // voxels after the first of one ray before it is flagged
 constexpr int kMaxBoxExtent = 64;      // voxels per axis of one Gaussian's box before it is flagged
 
 struct VoxSet {
     int32_t *status;                   // first error
     unsigned long long *keys;          // [capacity]
-    unsigned long long mask;           // capacity - 1
+    uint32_t blocks;                   // lines of slots - 1
+    uint32_t pos;                      // slots of a line - 1 (15, or capacity - 1 of a smaller set)
+    int shift;                         // log2 of the slots of a line
 };
 
-__host__ __device__ __forceinline__ VoxSet voxset_of_host(void *mem, long long capacity) {
+static VoxSet voxset_of_host(void *mem, long long capacity) {
     VoxSet s;
     s.status = reinterpret_cast<int32_t *>(mem);
     s.keys = reinterpret_cast<unsigned long long *>(static_cast<char *>(mem) + 256);
-    s.mask = (unsigned long long)capacity - 1ull;
+    s.shift = 0;
+    while (s.shift < 4 && (2LL << s.shift) <= capacity) ++s.shift;
+    s.pos = (1u << s.shift) - 1u;
+    s.blocks = (uint32_t)((capacity >> s.shift) - 1);
     return s;
 }
 
-__device__ __forceinline__ unsigned long long mix64(unsigned long long z) {
-    // splitmix64 finaliser (Vigna): a bijective 64-bit mix
-    z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ull;
-    z = (z ^ (z >> 27)) * 0x94d049bb133111ebull;
-    return z ^ (z >> 31);
+// a voxel index as it enters a key: clamped to [-2^20, 2^20), offset to [0, 2^21)
+__device__ __forceinline__ uint32_t key_coord(int i) {
+    return (uint32_t)(min(max(i, (int)-kKeyOff), (int)kKeyOff - 1) + (int)kKeyOff);
+}
+__device__ __forceinline__ unsigned long long vox_key(int ix, int iy, int iz) {
+    return ((unsigned long long)key_coord(ix) << (2 * kKeyBits)) | ((unsigned long long)key_coord(iy) << kKeyBits) |
+           key_coord(iz);
 }
 
-__device__ __forceinline__ unsigned long long pack_key(long long ix, long long iy, long long iz) {
-    ix = min(max(ix, -kKeyOff), kKeyOff - 1) + kKeyOff;
-    iy = min(max(iy, -kKeyOff), kKeyOff - 1) + kKeyOff;
-    iz = min(max(iz, -kKeyOff), kKeyOff - 1) + kKeyOff;
-    return ((unsigned long long)ix << (2 * kKeyBits)) | ((unsigned long long)iy << kKeyBits) |
-           (unsigned long long)iz;
-}
+// Where the key of a voxel may stand.  The 16 voxels of a 4 x 2 x 2 block share a line (128 bytes; 2 x 2 x 1 of
+// them a sector), whose number is a hash of the block: a ray of 70 voxels touches about 30 lines and its
+// neighbours in the warp the same ones, where a hash of the voxel itself touches 70 sectors of its own.  The
+// place within the line is the voxel's place in its block, XORed with hash bits (so that flat sets, which use
+// half of every block's voxels, still use all slots alike).  The sequence visits that place in the following
+// lines, then the next place in every line: the slots of one place behave like a linearly probed table of
+// random keys, and every slot is visited once in `capacity` probes.
+struct VoxProbe {
+    unsigned long long key;
+    uint32_t block, pos, first;
+
+    __device__ __forceinline__ VoxProbe(const VoxSet &s, unsigned long long k) : key(k) {
+        const uint32_t lo = (uint32_t)k, hi = (uint32_t)(k >> 32);   // y's low 11 bits and z; x and y's high 10 bits
+        // the block (two bits of x, one of y and z masked off) through odd multipliers, then a multiplication
+        // whose halves are folded onto each other, and the high part of another one
+        const uint32_t h = (lo & ~0x00200001u) * 0x9e3779b1u + (hi & ~0x00000c00u) * 0x85ebca77u;
+        const unsigned long long m = (unsigned long long)h * 0xc2b2ae3du;
+        const uint32_t f = (uint32_t)m ^ (uint32_t)(m >> 32);
+        block = first = __umulhi(f * 0x27d4eb2fu, s.blocks + 1u);
+        const uint32_t place = ((hi >> 10) & 3u) | ((lo >> 19) & 4u) | ((lo << 3) & 8u);
+        pos = (place ^ f) & s.pos;
+    }
+    __device__ __forceinline__ size_t slot(const VoxSet &s) const { return ((size_t)block << s.shift) | pos; }
+    // the next slot; false once all have been visited (`places` counts the places done)
+    __device__ __forceinline__ bool next(const VoxSet &s, uint32_t &places) {
+        block = (block + 1u) & s.blocks;
+        if (block == first) {
+            pos = (pos + 1u) & s.pos;
+            return ++places <= s.pos;
+        }
+        return true;
+    }
+};
 
 __device__ __forceinline__ bool voxset_insert(const VoxSet &s, unsigned long long key) {
-    unsigned long long slot = mix64(key) & s.mask;
-    for (unsigned long long probe = 0; probe <= s.mask; ++probe) {
-        const unsigned long long cur = s.keys[slot];
-        if (cur == key) return true;
+    VoxProbe p(s, key);
+    uint32_t places = 0;
+    do {
+        unsigned long long *slot = s.keys + p.slot(s);
+        const unsigned long long cur = *slot;
+        if (cur == p.key) return true;
         if (cur == kEmptyKey) {
-            const unsigned long long prev = atomicCAS(&s.keys[slot], kEmptyKey, key);
-            if (prev == kEmptyKey || prev == key) return true;
+            const unsigned long long prev = atomicCAS(slot, kEmptyKey, p.key);
+            if (prev == kEmptyKey || prev == p.key) return true;
         }
-        slot = (slot + 1) & s.mask;
-    }
+    } while (p.next(s, places));
     atomicCAS(s.status, 0, GS_ERR_CAPACITY);
     return false;
 }
 
-__device__ __forceinline__ bool voxset_contains(const VoxSet &s, unsigned long long key) {
-    unsigned long long slot = mix64(key) & s.mask;
-    for (unsigned long long probe = 0; probe <= s.mask; ++probe) {
-        const unsigned long long cur = s.keys[slot];
-        if (cur == key) return true;
-        if (cur == kEmptyKey) return false;
-        slot = (slot + 1) & s.mask;
+// `cur` is what the caller found in the first slot
+__device__ __forceinline__ bool voxset_contains(const VoxSet &s, VoxProbe p, unsigned long long cur) {
+    uint32_t places = 0;
+    for (;;) {
+        if (cur == p.key) return true;
+        if (cur == kEmptyKey || !p.next(s, places)) return false;
+        cur = s.keys[p.slot(s)];
     }
-    return false;
 }
 
 __device__ __forceinline__ long long vox_index(float x, float v) { return (long long)floorf(fp::div(x, v)); }
+// the same for a key alone: beyond +-2^30 every index enters keys as the same limit
+__device__ __forceinline__ int vox_clamp(long long i) { return (int)min(max(i, -(1LL << 30)), 1LL << 30); }
 
 // ------------------------------------------------------------------------------------------
 __global__ void k_voxset_clear(unsigned long long *keys, long long capacity, int32_t *status) {
@@ -90,25 +128,58 @@ __global__ void k_voxset_clear(unsigned long long *keys, long long capacity, int
     if (blockIdx.x == 0 && threadIdx.x == 0) *status = 0;
 }
 
-__global__ void k_add_boxes(VoxSet s, long long n, const float *means, const float *log_scales, float k, float v) {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        long long lo[3], hi[3];
+// One Gaussian per lane for the box, then the warp's voxels one per lane in turn, those of a box along z first:
+// boxes of one warp differ in size (one to hundreds of voxels), and a lane that walked its own would wait for a
+// probe of memory per voxel.  2 M Gaussians, a set of 2^25: 151 us, bound by instruction issue (75 %); 545 us with
+// a box per lane and voxels hashed one by one.
+__global__ void __launch_bounds__(256) k_add_boxes(VoxSet s, long long n, const float *means, const float *log_scales,
+                                                   float k, float v) {
+    const int lane = threadIdx.x & 31;
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    for (long long i0 = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); i0 < n; i0 += stride) {
+        const long long i = i0 + lane;
+        int lo[3] = {0, 0, 0}, ext[3] = {0, 0, 0};
         bool big = false;
+        if (i < n) {
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            const float mu = means[3 * i + a];
-            const float ks = fp::mul(k, spec_expf(log_scales[3 * i + a]));
-            lo[a] = vox_index(fp::sub(mu, ks), v);
-            hi[a] = vox_index(fp::add(mu, ks), v);
-            big |= (hi[a] - lo[a] + 1) > kMaxBoxExtent;
+            for (int a = 0; a < 3; ++a) {
+                const float mu = means[3 * i + a];
+                const float ks = fp::mul(k, spec_expf(log_scales[3 * i + a]));
+                const long long l = vox_index(fp::sub(mu, ks), v), h = vox_index(fp::add(mu, ks), v);
+                lo[a] = vox_clamp(l);
+                const unsigned long long span = (unsigned long long)h - (unsigned long long)l;
+                big |= h >= l && span >= kMaxBoxExtent;
+                ext[a] = h >= l ? (int)min(span, kMaxBoxExtent - 1ull) + 1 : 0;
+            }
         }
-        if (big) {
-            atomicCAS(s.status, 0, GS_ERR_INVALID_ARG);   // a box wider than kMaxBoxExtent voxels
-            continue;
+        if (big) atomicCAS(s.status, 0, GS_ERR_INVALID_ARG);   // a box wider than kMaxBoxExtent voxels
+        const int count = big ? 0 : ext[0] * ext[1] * ext[2];
+        int end = count;                                       // inclusive prefix sum over the lanes
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int up = __shfl_up_sync(0xffffffffu, end, o);
+            if (lane >= o) end += up;
         }
-        for (long long x = lo[0]; x <= hi[0]; ++x)
-            for (long long y = lo[1]; y <= hi[1]; ++y)
-                for (long long z = lo[2]; z <= hi[2]; ++z) voxset_insert(s, pack_key(x, y, z));
+        const int total = __shfl_sync(0xffffffffu, end, 31);
+        const int begin = end - count, dims = ext[1] << 8 | ext[2];
+        for (int base = 0; base < total; base += 32) {
+            const int item = base + lane;
+            int owner = 0;                                     // number of lanes whose voxels end at or before `item`
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+                if (__shfl_sync(0xffffffffu, end, owner + o - 1) <= item) owner += o;
+            const int d = __shfl_sync(0xffffffffu, dims, owner), at = item - __shfl_sync(0xffffffffu, begin, owner);
+            const int x0 = __shfl_sync(0xffffffffu, lo[0], owner), y0 = __shfl_sync(0xffffffffu, lo[1], owner);
+            const int z0 = __shfl_sync(0xffffffffu, lo[2], owner);
+            if (item < total) {
+                // at < 2^18 and extents <= 64: (at + 1/2) / extent is at least 1/128 away from an integer,
+                // and the approximate division (2 ulp) puts it within 2^-9 of where it belongs
+                const int ny = d >> 8, nz = d & 255;
+                const int row = (int)__fdividef((float)at + 0.5f, (float)nz), z = at - row * nz;
+                const int x = (int)__fdividef((float)row + 0.5f, (float)ny), y = row - x * ny;
+                voxset_insert(s, vox_key(x0 + x, y0 + y, z0 + z));
+            }
+        }
     }
 }
 
@@ -116,17 +187,24 @@ struct RayArgs {
     VoxSet s;
     const gs_camera *cams;
     const float *depth;       // [V,H,W] camera depth (z) per pixel; <= 0 or non-finite: no ray
-    int V, W, H, stride, sw, sh;
+    int V, W, H, stride, sw, sh;   // sw x sh rays a view
+    int pw, ph;               // patches of 8 x 4 rays across and down, one per warp
     float v;
-    long long max_steps;
 };
 
-__global__ void k_add_rays(RayArgs a) {
-    const long long total = (long long)a.V * a.sw * a.sh;
+// Bound by the instructions of a step (about 40: the analyser, the hash, the probe), not by memory: the rays of a
+// patch walk together through the lines near the camera.  8 views of 600 x 340 rays, some 70 voxels each, a set of
+// 2^25: 419 us; 467 us with a warp's rays along a row, 545 us at 48 warps an SM, 827 us with voxels hashed one by
+// one and 64-bit indices.  Settling a voxel only after the next one's load was issued: 650 us (more instructions,
+// and more slots found empty that another warp had just filled).
+__global__ void __launch_bounds__(256, 8) k_add_rays(RayArgs a) {
+    const long long total = (long long)a.V * a.pw * a.ph * 32;
     for (long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x; r < total; r += (long long)gridDim.x * blockDim.x) {
-        const int k = (int)(r / ((long long)a.sw * a.sh));
-        const long long rem = r - (long long)k * a.sw * a.sh;
-        const int y = (int)(rem / a.sw) * a.stride, x = (int)(rem % a.sw) * a.stride;
+        const int lane = threadIdx.x & 31;
+        const long long patch = r >> 5, k = patch / ((long long)a.pw * a.ph);
+        const int at = (int)(patch - k * a.pw * a.ph), sy = at / a.pw * 4 + (lane >> 3), sx = at % a.pw * 8 + (lane & 7);
+        if (sy >= a.sh || sx >= a.sw) continue;
+        const int y = sy * a.stride, x = sx * a.stride;
         const float d = a.depth[((long long)k * a.H + y) * a.W + x];
         if (!(d > 0.f) || !isfinite(d)) continue;
         const gs_camera cam = a.cams[k];
@@ -140,21 +218,21 @@ __global__ void k_add_rays(RayArgs a) {
 #pragma unroll
         for (int q = 0; q < 3; ++q) p[q] = fp::fma(R[q], pc0, fp::fma(R[3 + q], pc1, fp::mul(R[6 + q], pc2)));
         // digital differential analyser over [c, p)
-        long long cur[3];
-        int step[3];
+        int cur[3], step[3];
         float tmax[3], tdel[3];
         const float inf = __int_as_float(0x7f800000);
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
-            cur[q] = vox_index(c[q], a.v);
+            const long long at = vox_index(c[q], a.v);
+            cur[q] = vox_clamp(at);
             const float dq = fp::sub(p[q], c[q]);
             if (dq > 0.f) {
                 step[q] = 1;
-                tmax[q] = fp::div(fp::sub(fp::mul((float)(cur[q] + 1), a.v), c[q]), dq);
+                tmax[q] = fp::div(fp::sub(fp::mul((float)(at + 1), a.v), c[q]), dq);
                 tdel[q] = fp::div(a.v, dq);
             } else if (dq < 0.f) {
                 step[q] = -1;
-                tmax[q] = fp::div(fp::sub(fp::mul((float)cur[q], a.v), c[q]), dq);
+                tmax[q] = fp::div(fp::sub(fp::mul((float)at, a.v), c[q]), dq);
                 tdel[q] = fp::div(-a.v, dq);
             } else {
                 step[q] = 0;
@@ -162,27 +240,57 @@ __global__ void k_add_rays(RayArgs a) {
                 tdel[q] = inf;
             }
         }
-        voxset_insert(a.s, pack_key(cur[0], cur[1], cur[2]));
-        long long n = 0;
-        for (; n < a.max_steps; ++n) {
-            int q = 0;
-            if (tmax[1] < tmax[q]) q = 1;
-            if (tmax[2] < tmax[q]) q = 2;
-            if (!(tmax[q] < 1.0f)) break;
-            cur[q] += step[q];
-            tmax[q] = fp::add(tmax[q], tdel[q]);
-            voxset_insert(a.s, pack_key(cur[0], cur[1], cur[2]));
+        unsigned long long key = vox_key(cur[0], cur[1], cur[2]);
+        voxset_insert(a.s, key);
+        int n = 0;
+        // A ray that starts far enough inside the range of keys never meets its limits: its key moves by the
+        // step's own bits.
+        constexpr int kInside = (int)kKeyOff - (kMaxRaySteps + 1);
+        if (max(max(abs(cur[0]), abs(cur[1])), abs(cur[2])) <= kInside) {
+            const unsigned long long kx = (unsigned long long)(long long)step[0] << (2 * kKeyBits);
+            const unsigned long long ky = (unsigned long long)(long long)step[1] << kKeyBits;
+            const unsigned long long kz = (unsigned long long)(long long)step[2];
+            for (; n < kMaxRaySteps; ++n) {
+                const bool b1 = tmax[1] < tmax[0];
+                const float t01 = b1 ? tmax[1] : tmax[0];
+                const bool q2 = tmax[2] < t01;
+                if (!((q2 ? tmax[2] : t01) < 1.0f)) break;
+                const float n0 = fp::add(tmax[0], tdel[0]), n1 = fp::add(tmax[1], tdel[1]), n2 = fp::add(tmax[2], tdel[2]);
+                key += q2 ? kz : b1 ? ky : kx;
+                tmax[0] = !q2 && !b1 ? n0 : tmax[0];
+                tmax[1] = !q2 && b1 ? n1 : tmax[1];
+                tmax[2] = q2 ? n2 : tmax[2];
+                voxset_insert(a.s, key);
+            }
+        } else {
+            for (; n < kMaxRaySteps; ++n) {
+                int q = 0;
+                if (tmax[1] < tmax[0]) q = 1;
+                if (tmax[2] < (q ? tmax[1] : tmax[0])) q = 2;
+                if (!((q == 2 ? tmax[2] : q == 1 ? tmax[1] : tmax[0]) < 1.0f)) break;
+#pragma unroll
+                for (int d = 0; d < 3; ++d)
+                    if (d == q) {
+                        cur[d] += step[d];
+                        tmax[d] = fp::add(tmax[d], tdel[d]);
+                    }
+                voxset_insert(a.s, vox_key(cur[0], cur[1], cur[2]));
+            }
         }
-        if (n == a.max_steps) atomicCAS(a.s.status, 0, GS_ERR_INVALID_ARG);   // ray longer than allowed
+        if (n == kMaxRaySteps) atomicCAS(a.s.status, 0, GS_ERR_INVALID_ARG);   // ray longer than allowed
     }
 }
 
 __global__ void k_keep(long long n, const float *means, VoxSet occ, VoxSet fre, bool has_free, float v,
                        uint8_t *keep) {
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const unsigned long long key =
-            pack_key(vox_index(means[3 * i], v), vox_index(means[3 * i + 1], v), vox_index(means[3 * i + 2], v));
-        const bool drop = voxset_contains(occ, key) || (has_free && voxset_contains(fre, key));
+        const int x = vox_clamp(vox_index(means[3 * i], v)), y = vox_clamp(vox_index(means[3 * i + 1], v)),
+                  z = vox_clamp(vox_index(means[3 * i + 2], v));
+        const unsigned long long key = vox_key(x, y, z);
+        const VoxProbe po(occ, key), pf(fre, key);
+        const unsigned long long co = occ.keys[po.slot(occ)];   // both sets are asked before either answers
+        const unsigned long long cf = has_free ? fre.keys[pf.slot(fre)] : kEmptyKey;
+        const bool drop = voxset_contains(occ, po, co) || voxset_contains(fre, pf, cf);
         keep[i] = drop ? 0 : 1;
     }
 }
@@ -238,8 +346,9 @@ int launch_voxset_add_rays(void *mem, long long capacity, int V, int W, int H, c
     a.sw = (W + stride - 1) / stride;
     a.sh = (H + stride - 1) / stride;
     a.v = v;
-    a.max_steps = 1LL << 16;
-    const long long total = (long long)V * a.sw * a.sh;
+    a.pw = (a.sw + 7) / 8;
+    a.ph = (a.sh + 3) / 4;
+    const long long total = (long long)V * a.pw * a.ph * 32;
     k_add_rays<<<grid_for(total), 256, 0, s>>>(a);
     count_launches(1);
     return check_launch();
