@@ -18,7 +18,11 @@ def _ptr(t):
 
 
 def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    """The current stream's handle, without the Stream object of torch.cuda.current_stream() (0.3 us for 3 us, six
+    times in a differentiated render)."""
+    if not torch.cuda.is_initialized():
+        return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return C.c_void_p(torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()))
 
 
 def default_params(**over) -> L.gs_params:
@@ -60,8 +64,9 @@ class Gaussians:
 
 
 def zeros_like_grads(g: Gaussians) -> Gaussians:
-    return Gaussians(*[torch.zeros_like(getattr(g, k)) for k in ("means", "log_scales", "quats", "opacities",
-                                                                  "colors")])
+    out = [torch.empty_like(getattr(g, k)) for k in ("means", "log_scales", "quats", "opacities", "colors")]
+    torch._foreach_zero_(out)   # one launch for the five (18 us of host time for 54)
+    return Gaussians(*out)
 
 
 def cameras_tensor(cameras, device="cuda") -> torch.Tensor:
