@@ -471,7 +471,10 @@ __global__ void __launch_bounds__(kSortThreads) k_onesweep(SweepArgs a) {
 // ------------------------------------------------------------------------------------------
 // A warp per 32 keys: a lane per key finds the range borders, the pair's slot and the value, then the
 // 96 16-byte parts of the 32 records are copied by consecutive lanes (a record's three parts by three
-// neighbouring lanes, so every store instruction writes 512 contiguous bytes).
+// neighbouring lanes, so every store instruction writes 512 contiguous bytes).  The lists are streamed past the
+// L2 (64 B a key written once): it is the records of the view in hand, gathered about three times each, that
+// should stay there.  The step of 64 views of 4 M
+// Gaussians (194 M keys) goes from 61.3 to 59.3 ms with it; lists that fit the L2 neither gain nor lose.
 constexpr int kRecThreads = 256;
 __global__ void __launch_bounds__(kRecThreads) k_records(BinArgs a) {
     const unsigned long long K = min(a.st->num_keys, (unsigned long long)a.cap);
@@ -494,7 +497,7 @@ __global__ void __launch_bounds__(kRecThreads) k_records(BinArgs a) {
             } else {
                 if (g != prev) a.ranges[2 * (size_t)g] = (uint32_t)i;
                 if (g != next) a.ranges[2 * (size_t)g + 1] = (uint32_t)(i + 1);
-                vout[i] = f;
+                __stcs(vout + i, f);
                 sl = a.slot[f];
                 if (sl >= (unsigned long long)a.vcap) {         // only after an earlier recorded failure
                     record_error(a.st, GS_ERR_DEVICE_FAULT, 8);
@@ -509,10 +512,10 @@ __global__ void __launch_bounds__(kRecThreads) k_records(BinArgs a) {
             if (se != kNoSlot) {
                 float4 r = a.proj[3 * (size_t)se + part];
                 if (part == 1) {
-                    kout[i0 + e] = ((unsigned long long)ge << 32) | __float_as_uint(r.z);
+                    __stcs(reinterpret_cast<unsigned long long *>(kout) + i0 + e, ((unsigned long long)ge << 32) | __float_as_uint(r.z));
                     r.w = __uint_as_float(se);   // the radius (used only by the emission) gives way to the slot
                 }
-                a.srec[3 * i0 + q] = r;
+                __stcs(a.srec + 3 * i0 + q, r);
             }
         }
     }
