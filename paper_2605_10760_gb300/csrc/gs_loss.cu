@@ -134,32 +134,32 @@ static SsimTaps make_taps() {
     return t;
 }
 
-// Both passes: 256 threads per 32 x 32 output tile.  The inputs are fetched 16 bytes at a time where the
-// planes allow it: 42 rows of 48 columns, from 8 left of the tile, so that every group of four is in or out as
-// a whole.  The horizontal filter gives a thread four adjacent columns of one row, so it loads 16 inputs for
-// four outputs; the vertical filter four rows of one column.  Values that take the same taps are the two
-// components of packed FP32x2 arithmetic: pass 1 filters (x, y) and (x^2, y^2) packed and x y alone, pass 2
-// (dS/dmu_x, dS/dE[x^2]) packed and dS/dE[xy] alone.  (The SSIM map's mean enters an FP64 loss and its bias
+// Both passes: 256 threads walk a strip of 32 columns down `seg` rows, 32 rows a step.  The inputs of a step are
+// fetched 16 bytes at a time where the planes allow it: 48 columns, from 8 left of the strip, so that every group
+// of four is in or out as a whole.  The horizontal filter gives a thread four adjacent columns of one row, so it
+// loads 16 inputs for four outputs; the vertical filter four rows of one column.  The last ten filtered rows of a
+// step are the first of the next, and the sums are reduced once per strip.  Values that take the same taps are
+// the two components of packed FP32x2 arithmetic: pass 1 filters (x, y) and (x^2, y^2) packed and x y alone, pass
+// 2 (dS/dmu_x, dS/dE[x^2]) packed and dS/dE[xy] alone.  (The SSIM map's mean enters an FP64 loss and its bias
 // comes from the rounding of these sums, so their operations are part of the result: taps in ascending order,
 // w x rounded before it is added or meets its second factor.)  The pitches below and the order of the lanes in
 // the horizontal filter (hlane) keep every 16-byte shared access of eight lanes on 32 different banks.
-// 8 views of 1200 x 680 (19.6 M samples): pass 1 213 us (70 % of the issue slots; 392 MB take 58 us), pass 2
-// 173 us (63 %; 470 MB, 69 us); with one sample per load and scalar arithmetic 318 us and 279 us, plus 47 us
-// for a pass of its own for |x - y|.  The scalar
-// loads of other widths or alignments cost the 42 x 42 tile 7 guarded loads a thread instead of 2.
+// 8 views of 1200 x 680 (19.6 M samples): pass 1 187 us (68 % of the issue slots; 392 MB take 58 us), pass 2 142 us
+// (62 %; 470 MB, 69 us); tiles of 32 x 32 on their own 213 and 173 us; with one sample per load and scalar
+// arithmetic 318 and 279 us, plus 47 us for a pass of its own for |x - y|.
 constexpr int kSVR = 4;            // rows per thread in the vertical filter, columns in the horizontal one
-constexpr int kSC = 48;            // input columns, the tile's own from kSL
+constexpr int kSC = 48;            // input columns, the strip's own from kSL
 constexpr int kSL = 8;
-constexpr int kHItems = (kSI + 3) / 4 * 32;   // (row, column group) pairs of the horizontal filter, padded
+constexpr int kHalo = 2 * kR;      // filtered rows that two steps share
 
 struct __align__(16) Ssim1Smem {
-    float2 xy[kSI][kSC + 2];
+    float2 xy[kSB][kSC + 2];
     float4 h[kSI][kSB + 4];        // filtered x, y, x^2, y^2 of column c at c ^ (c >> 2)
     float hxy[kSI][kSB + 8];       // filtered x y, likewise
 };
 struct __align__(16) Ssim2Smem {
-    float2 a[kSI][kSC + 2];        // dS/dmu_x, dS/dE[x^2]
-    float b[kSI][kSC];             // dS/dE[xy]
+    float2 a[kSB][kSC + 2];        // dS/dmu_x, dS/dE[x^2]
+    float b[kSB][kSC];             // dS/dE[xy]
     float2 ha[kSI][kSB + 2];
     float hb[kSI][kSB + 16];
 };
@@ -206,82 +206,8 @@ __device__ __forceinline__ void block_add2(float2 a, float2 b, double *pa, doubl
     }
 }
 
-// Pass 1 of one tile of one plane: x, y (x optionally as fl(fl(ea x) + eb)), zero padding; the blurred
-// moments, the SSIM map and |x - y| summed over the thread's share, and the three per-pixel derivatives
-// dS/dmu_x, dS/dE[x^2], dS/dE[xy] (scaled by inv_n) written for pass 2.
-template <bool EXPO, bool VEC>
-__device__ __forceinline__ void ssim_pass1_tile(Ssim1Smem &sm, int W, int H, const float *xp, const float *yp, float ea,
-                                                float eb, const SsimTaps &tp, float inv_n, float *dmu, float *dexx,
-                                                float *dexy, float2 &s_ssim, float2 &s_l1) {
-    const int x0 = blockIdx.x * kSB - kSL, y0 = blockIdx.y * kSB - kR;
-    s_ssim = s_l1 = make_float2(0.f, 0.f);
-    float4 xv[2], yv[2];
-#pragma unroll
-    for (int part = 0; part < 2; ++part) {   // every load before the first store
-        const int i = threadIdx.x + 256 * part, r = i / (kSC / 4), c = (i - r * (kSC / 4)) * 4;
-        const int gx = x0 + c, gy = y0 + r;
-        xv[part] = yv[part] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (r < kSI && gy >= 0 && gy < H) {
-            xv[part] = load4<VEC>(xp + (long long)gy * W, gx, W);
-            yv[part] = load4<VEC>(yp + (long long)gy * W, gx, W);
-            if (EXPO) {   // the padding stays zero
-                float4 &x = xv[part];
-                if (gx >= 0 && gx < W) x.x = fp::add(fp::mul(ea, x.x), eb);
-                if (VEC ? gx >= 0 && gx < W : gx + 1 >= 0 && gx + 1 < W) x.y = fp::add(fp::mul(ea, x.y), eb);
-                if (VEC ? gx >= 0 && gx < W : gx + 2 >= 0 && gx + 2 < W) x.z = fp::add(fp::mul(ea, x.z), eb);
-                if (VEC ? gx >= 0 && gx < W : gx + 3 >= 0 && gx + 3 < W) x.w = fp::add(fp::mul(ea, x.w), eb);
-            }
-        }
-    }
-#pragma unroll
-    for (int part = 0; part < 2; ++part) {
-        const int i = threadIdx.x + 256 * part, r = i / (kSC / 4), c = (i - r * (kSC / 4)) * 4;
-        if (r >= kSI) break;
-        float4 *d = reinterpret_cast<float4 *>(&sm.xy[r][c]);
-        d[0] = make_float4(xv[part].x, yv[part].x, xv[part].y, yv[part].y);
-        d[1] = make_float4(xv[part].z, yv[part].z, xv[part].w, yv[part].w);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < kHItems; i += 256) {
-        const int r = hlane_row(i), t = hlane_group(i);
-        if (r >= kSI) continue;
-        float2 m[kSVR], q[kSVR];
-        float p[kSVR];
-#pragma unroll
-        for (int j = 0; j < kSVR; ++j) {
-            m[j] = q[j] = make_float2(0.f, 0.f);
-            p[j] = 0.f;
-        }
-        // output column 4 t + j takes inputs 4 t + j + kSL - kR + (0 .. 2 kR)
-        const float4 *src = reinterpret_cast<const float4 *>(&sm.xy[r][4 * t]);
-        constexpr int kFirst = kSL - kR;
-#pragma unroll
-        for (int u = kFirst / 2; u <= (kFirst + kSVR - 1 + 2 * kR) / 2; ++u) {
-            const float4 f = src[u];
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const int k = 2 * u + e - kFirst;
-                const float2 v = e ? make_float2(f.z, f.w) : make_float2(f.x, f.y);
-#pragma unroll
-                for (int j = 0; j < kSVR; ++j) {
-                    if (k - j >= 0 && k - j <= 2 * kR) {
-                        const float2 wv = fp2::mul(fp2::splat(tp.w[k - j]), v);
-                        m[j] = fp2::add(wv, m[j]);
-                        q[j] = fp2::fma(wv, v, q[j]);
-                        p[j] = fmaf(wv.x, v.y, p[j]);
-                    }
-                }
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < kSVR; ++j) {
-            const int c = (4 * t + j) ^ t;
-            sm.h[r][c] = make_float4(m[j].x, m[j].y, q[j].x, q[j].y);
-            sm.hxy[r][c] = p[j];
-        }
-    }
-    __syncthreads();
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, tc = tx ^ (tx >> 2);
+// One row's four columns t of the horizontal filters, from row r of the inputs into row d of the filtered rows
+__device__ __forceinline__ void ssim1_hfilter(Ssim1Smem &sm, const SsimTaps &tp, int r, int t, int d) {
     float2 m[kSVR], q[kSVR];
     float p[kSVR];
 #pragma unroll
@@ -289,131 +215,250 @@ __device__ __forceinline__ void ssim_pass1_tile(Ssim1Smem &sm, int W, int H, con
         m[j] = q[j] = make_float2(0.f, 0.f);
         p[j] = 0.f;
     }
+    // output column 4 t + j takes inputs 4 t + j + kSL - kR + (0 .. 2 kR)
+    const float4 *src = reinterpret_cast<const float4 *>(&sm.xy[r][4 * t]);
+    constexpr int kFirst = kSL - kR;
 #pragma unroll
-    for (int k = 0; k < kSVR + 2 * kR; ++k) {
-        const float4 v = sm.h[ty * kSVR + k][tc];
-        const float vp = sm.hxy[ty * kSVR + k][tc];
+    for (int u = kFirst / 2; u <= (kFirst + kSVR - 1 + 2 * kR) / 2; ++u) {
+        const float4 f = src[u];
 #pragma unroll
-        for (int j = 0; j < kSVR; ++j) {
-            if (k - j >= 0 && k - j <= 2 * kR) {
-                const float2 w = fp2::splat(tp.w[k - j]);
-                m[j] = fp2::fma(w, make_float2(v.x, v.y), m[j]);
-                q[j] = fp2::fma(w, make_float2(v.z, v.w), q[j]);
-                p[j] = fmaf(tp.w[k - j], vp, p[j]);
-            }
-        }
-    }
-    const int gx = blockIdx.x * kSB + tx, gy0 = blockIdx.y * kSB + ty * kSVR;
-    if (gx >= W) return;
+        for (int e = 0; e < 2; ++e) {
+            const int k = 2 * u + e - kFirst;
+            const float2 v = e ? make_float2(f.z, f.w) : make_float2(f.x, f.y);
 #pragma unroll
-    for (int j = 0; j < kSVR; ++j) {
-        if (gy0 + j >= H) break;
-        const float mx = m[j].x, my = m[j].y, exx = q[j].x, eyy = q[j].y, exy = p[j];
-        const float vx = exx - mx * mx, vy = eyy - my * my, cxy = exy - mx * my;
-        const float A1 = 2.f * mx * my + kC1, A2 = 2.f * cxy + kC2;
-        const float B1 = mx * mx + my * my + kC1, B2 = vx + vy + kC2;
-        const float iB = 1.f / (B1 * B2), iB1 = iB * B2, iB2 = iB * B1;
-        const float S = A1 * A2 * iB;
-        const float2 v = sm.xy[ty * kSVR + j + kR][tx + kSL];
-        add_to_pair(s_ssim, S);
-        add_to_pair(s_l1, fabsf(v.x - v.y));
-        const long long o = (long long)(gy0 + j) * W + gx;
-        dmu[o] = inv_n * ((2.f * my * A2 - 2.f * my * A1) * iB - S * (2.f * mx * iB1 - 2.f * mx * iB2));
-        dexx[o] = inv_n * (-S * iB2);
-        dexy[o] = inv_n * (2.f * A1 * iB);
-    }
-}
-
-// Pass 2 of one tile: the three derivative maps blurred (the adjoint of a zero-padded symmetric
-// blur is the same blur); ga = (blur(dS/dmu_x), blur(dS/dE[x^2])), gb = blur(dS/dE[xy]) for the thread's
-// kSVR outputs.
-template <bool VEC>
-__device__ __forceinline__ void ssim_pass2_tile(Ssim2Smem &sm, int W, int H, const float *dmu, const float *dexx,
-                                                const float *dexy, const SsimTaps &tp, float2 (&ga)[kSVR],
-                                                float (&gb)[kSVR]) {
-    const int x0 = blockIdx.x * kSB - kSL, y0 = blockIdx.y * kSB - kR;
-    float4 v0[2], v1[2], v2[2];
-#pragma unroll
-    for (int part = 0; part < 2; ++part) {
-        const int i = threadIdx.x + 256 * part, r = i / (kSC / 4), c = (i - r * (kSC / 4)) * 4;
-        const int gx = x0 + c, gy = y0 + r;
-        v0[part] = v1[part] = v2[part] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (r < kSI && gy >= 0 && gy < H) {
-            const long long o = (long long)gy * W;
-            v0[part] = load4<VEC>(dmu + o, gx, W);
-            v1[part] = load4<VEC>(dexx + o, gx, W);
-            v2[part] = load4<VEC>(dexy + o, gx, W);
-        }
-    }
-#pragma unroll
-    for (int part = 0; part < 2; ++part) {
-        const int i = threadIdx.x + 256 * part, r = i / (kSC / 4), c = (i - r * (kSC / 4)) * 4;
-        if (r >= kSI) break;
-        float4 *d = reinterpret_cast<float4 *>(&sm.a[r][c]);
-        d[0] = make_float4(v0[part].x, v1[part].x, v0[part].y, v1[part].y);
-        d[1] = make_float4(v0[part].z, v1[part].z, v0[part].w, v1[part].w);
-        *reinterpret_cast<float4 *>(&sm.b[r][c]) = v2[part];
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < kHItems; i += 256) {
-        const int r = hlane_row(i), t = hlane_group(i);
-        if (r >= kSI) continue;
-        float2 a[kSVR];
-        float b[kSVR];
-#pragma unroll
-        for (int j = 0; j < kSVR; ++j) {
-            a[j] = make_float2(0.f, 0.f);
-            b[j] = 0.f;
-        }
-        const float4 *sa = reinterpret_cast<const float4 *>(&sm.a[r][4 * t]);
-        const float4 *sb = reinterpret_cast<const float4 *>(&sm.b[r][4 * t]);
-        constexpr int kFirst = kSL - kR;
-#pragma unroll
-        for (int u = 0; u <= (kFirst + kSVR - 1 + 2 * kR) / 4; ++u) {
-            const float4 f0 = sa[2 * u], f1 = sa[2 * u + 1], fb = sb[u];
-            const float2 va[4] = {make_float2(f0.x, f0.y), make_float2(f0.z, f0.w), make_float2(f1.x, f1.y),
-                                  make_float2(f1.z, f1.w)};
-            const float vb[4] = {fb.x, fb.y, fb.z, fb.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int k = 4 * u + e - kFirst;
-#pragma unroll
-                for (int j = 0; j < kSVR; ++j) {
-                    if (k - j >= 0 && k - j <= 2 * kR) {
-                        a[j] = fp2::fma(fp2::splat(tp.w[k - j]), va[e], a[j]);
-                        b[j] = fmaf(tp.w[k - j], vb[e], b[j]);
-                    }
+            for (int j = 0; j < kSVR; ++j) {
+                if (k - j >= 0 && k - j <= 2 * kR) {
+                    const float2 wv = fp2::mul(fp2::splat(tp.w[k - j]), v);
+                    m[j] = fp2::add(wv, m[j]);
+                    q[j] = fp2::fma(wv, v, q[j]);
+                    p[j] = fmaf(wv.x, v.y, p[j]);
                 }
             }
         }
-        float4 *da = reinterpret_cast<float4 *>(&sm.ha[r][4 * t]);
-        da[0] = make_float4(a[0].x, a[0].y, a[1].x, a[1].y);
-        da[1] = make_float4(a[2].x, a[2].y, a[3].x, a[3].y);
-        *reinterpret_cast<float4 *>(&sm.hb[r][4 * t]) = make_float4(b[0], b[1], b[2], b[3]);
     }
-    __syncthreads();
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
 #pragma unroll
     for (int j = 0; j < kSVR; ++j) {
-        ga[j] = make_float2(0.f, 0.f);
-        gb[j] = 0.f;
+        const int c = (4 * t + j) ^ t;
+        sm.h[d][c] = make_float4(m[j].x, m[j].y, q[j].x, q[j].y);
+        sm.hxy[d][c] = p[j];
     }
+}
+
+__device__ __forceinline__ void ssim2_hfilter(Ssim2Smem &sm, const SsimTaps &tp, int r, int t, int d) {
+    float2 a[kSVR];
+    float b[kSVR];
 #pragma unroll
-    for (int k = 0; k < kSVR + 2 * kR; ++k) {
-        const float2 va = sm.ha[ty * kSVR + k][tx];
-        const float vb = sm.hb[ty * kSVR + k][tx];
+    for (int j = 0; j < kSVR; ++j) {
+        a[j] = make_float2(0.f, 0.f);
+        b[j] = 0.f;
+    }
+    const float4 *sa = reinterpret_cast<const float4 *>(&sm.a[r][4 * t]);
+    const float4 *sb = reinterpret_cast<const float4 *>(&sm.b[r][4 * t]);
+    constexpr int kFirst = kSL - kR;
+#pragma unroll
+    for (int u = 0; u <= (kFirst + kSVR - 1 + 2 * kR) / 4; ++u) {
+        const float4 f0 = sa[2 * u], f1 = sa[2 * u + 1], fb = sb[u];
+        const float2 va[4] = {make_float2(f0.x, f0.y), make_float2(f0.z, f0.w), make_float2(f1.x, f1.y),
+                              make_float2(f1.z, f1.w)};
+        const float vb[4] = {fb.x, fb.y, fb.z, fb.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int k = 4 * u + e - kFirst;
+#pragma unroll
+            for (int j = 0; j < kSVR; ++j) {
+                if (k - j >= 0 && k - j <= 2 * kR) {
+                    a[j] = fp2::fma(fp2::splat(tp.w[k - j]), va[e], a[j]);
+                    b[j] = fmaf(tp.w[k - j], vb[e], b[j]);
+                }
+            }
+        }
+    }
+    float4 *da = reinterpret_cast<float4 *>(&sm.ha[d][4 * t]);
+    da[0] = make_float4(a[0].x, a[0].y, a[1].x, a[1].y);
+    da[1] = make_float4(a[2].x, a[2].y, a[3].x, a[3].y);
+    *reinterpret_cast<float4 *>(&sm.hb[d][4 * t]) = make_float4(b[0], b[1], b[2], b[3]);
+}
+
+// Pass 1 of a strip of one plane, rows [y_begin, y_end): x, y (x optionally as fl(fl(ea x) + eb)), zero padding;
+// the blurred moments, the SSIM map and |x - y| summed over the thread's share, and the three per-pixel
+// derivatives dS/dmu_x, dS/dE[x^2], dS/dE[xy] (scaled by inv_n) written for pass 2.
+template <bool EXPO, bool VEC>
+__device__ __forceinline__ void ssim_pass1_strip(Ssim1Smem &sm, int W, int H, const float *xp, const float *yp, float ea,
+                                                 float eb, const SsimTaps &tp, float inv_n, float *dmu, float *dexx,
+                                                 float *dexy, int y_begin, int y_end, float2 &s_ssim, float2 &s_l1) {
+    const int x0 = blockIdx.x * kSB - kSL;
+    const int hr = hlane_row(threadIdx.x), ht = hlane_group(threadIdx.x);
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, tc = tx ^ (tx >> 2);
+    const int gx = blockIdx.x * kSB + tx;
+    s_ssim = s_l1 = make_float2(0.f, 0.f);
+    for (int y0 = y_begin - kSB; y0 < y_end; y0 += kSB) {   // the first step only makes the ten rows above the strip
+        const bool lead = y0 < y_begin;
+        const int rows = lead ? kHalo : kSB, first = lead ? y_begin - kR : y0 + kR;
+        float4 xv[2], yv[2];
+#pragma unroll
+        for (int part = 0; part < 2; ++part) {   // every load before the first store
+            const int i = threadIdx.x + 256 * part, r = i / (kSC / 4), c = (i - r * (kSC / 4)) * 4;
+            const int lx = x0 + c, ly = first + r;
+            xv[part] = yv[part] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (r < rows && ly >= 0 && ly < H) {
+                xv[part] = load4<VEC>(xp + (long long)ly * W, lx, W);
+                yv[part] = load4<VEC>(yp + (long long)ly * W, lx, W);
+                if (EXPO) {   // the padding stays zero
+                    float4 &x = xv[part];
+                    if (lx >= 0 && lx < W) x.x = fp::add(fp::mul(ea, x.x), eb);
+                    if (VEC ? lx >= 0 && lx < W : lx + 1 >= 0 && lx + 1 < W) x.y = fp::add(fp::mul(ea, x.y), eb);
+                    if (VEC ? lx >= 0 && lx < W : lx + 2 >= 0 && lx + 2 < W) x.z = fp::add(fp::mul(ea, x.z), eb);
+                    if (VEC ? lx >= 0 && lx < W : lx + 3 >= 0 && lx + 3 < W) x.w = fp::add(fp::mul(ea, x.w), eb);
+                }
+                if (c >= kSL && c < kSL + kSB && ly >= y_begin && ly < y_end) {   // the strip's own (zeros beyond W)
+                    add_to_pair(s_l1, fabsf(xv[part].x - yv[part].x));
+                    add_to_pair(s_l1, fabsf(xv[part].y - yv[part].y));
+                    add_to_pair(s_l1, fabsf(xv[part].z - yv[part].z));
+                    add_to_pair(s_l1, fabsf(xv[part].w - yv[part].w));
+                }
+            }
+        }
+#pragma unroll
+        for (int part = 0; part < 2; ++part) {
+            const int i = threadIdx.x + 256 * part, r = i / (kSC / 4), c = (i - r * (kSC / 4)) * 4;
+            if (r >= rows) break;
+            float4 *d = reinterpret_cast<float4 *>(&sm.xy[r][c]);
+            d[0] = make_float4(xv[part].x, yv[part].x, xv[part].y, yv[part].y);
+            d[1] = make_float4(xv[part].z, yv[part].z, xv[part].w, yv[part].w);
+        }
+        __syncthreads();   // inputs stored; the last step's vertical filter is done
+        if (lead) {
+            if (hr < kHalo) ssim1_hfilter(sm, tp, hr, ht, hr);
+            __syncthreads();
+            continue;
+        }
+        if (y0 > y_begin) {
+            for (int i = threadIdx.x; i < kHalo * kSB; i += 256) {
+                const int r = i / kSB, c = i % kSB;
+                sm.h[r][c] = sm.h[kSB + r][c];
+                sm.hxy[r][c] = sm.hxy[kSB + r][c];
+            }
+            __syncthreads();
+        }
+        ssim1_hfilter(sm, tp, hr, ht, kHalo + hr);
+        __syncthreads();
+        float2 m[kSVR], q[kSVR];
+        float p[kSVR];
 #pragma unroll
         for (int j = 0; j < kSVR; ++j) {
-            if (k - j >= 0 && k - j <= 2 * kR) {
-                ga[j] = fp2::fma(fp2::splat(tp.w[k - j]), va, ga[j]);
-                gb[j] = fmaf(tp.w[k - j], vb, gb[j]);
+            m[j] = q[j] = make_float2(0.f, 0.f);
+            p[j] = 0.f;
+        }
+#pragma unroll
+        for (int k = 0; k < kSVR + 2 * kR; ++k) {
+            const float4 v = sm.h[ty * kSVR + k][tc];
+            const float vp = sm.hxy[ty * kSVR + k][tc];
+#pragma unroll
+            for (int j = 0; j < kSVR; ++j) {
+                if (k - j >= 0 && k - j <= 2 * kR) {
+                    const float2 w = fp2::splat(tp.w[k - j]);
+                    m[j] = fp2::fma(w, make_float2(v.x, v.y), m[j]);
+                    q[j] = fp2::fma(w, make_float2(v.z, v.w), q[j]);
+                    p[j] = fmaf(tp.w[k - j], vp, p[j]);
+                }
             }
+        }
+        const int gy0 = y0 + ty * kSVR;
+#pragma unroll
+        for (int j = 0; j < kSVR; ++j) {
+            if (gx >= W || gy0 + j >= y_end) break;
+            const float mx = m[j].x, my = m[j].y, exx = q[j].x, eyy = q[j].y, exy = p[j];
+            const float vx = exx - mx * mx, vy = eyy - my * my, cxy = exy - mx * my;
+            const float A1 = 2.f * mx * my + kC1, A2 = 2.f * cxy + kC2;
+            const float B1 = mx * mx + my * my + kC1, B2 = vx + vy + kC2;
+            const float iB = 1.f / (B1 * B2), iB1 = iB * B2, iB2 = iB * B1;
+            const float S = A1 * A2 * iB;
+            add_to_pair(s_ssim, S);
+            const long long o = (long long)(gy0 + j) * W + gx;
+            dmu[o] = inv_n * ((2.f * my * A2 - 2.f * my * A1) * iB - S * (2.f * mx * iB1 - 2.f * mx * iB2));
+            dexx[o] = inv_n * (-S * iB2);
+            dexy[o] = inv_n * (2.f * A1 * iB);
         }
     }
 }
 
-// the images at a thread's outputs, asked for before pass 2 waits for its tile (8 views of 1200 x 680: 235 us
-// with these loads after the filter, 173 us before it)
+// Pass 2 of a strip: the three derivative maps blurred (the adjoint of a zero-padded symmetric blur is the same
+// blur).  Per step, before(y) is called ahead of the loads and after(y, ga, gb) with
+// ga = (blur(dS/dmu_x), blur(dS/dE[x^2])) and gb = blur(dS/dE[xy]) of the thread's kSVR outputs, rows y ...
+template <bool VEC, typename Before, typename After>
+__device__ __forceinline__ void ssim_pass2_strip(Ssim2Smem &sm, int W, int H, const float *dmu, const float *dexx,
+                                                 const float *dexy, const SsimTaps &tp, int y_begin, int y_end,
+                                                 Before before, After after) {
+    const int x0 = blockIdx.x * kSB - kSL;
+    const int hr = hlane_row(threadIdx.x), ht = hlane_group(threadIdx.x);
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    for (int y0 = y_begin - kSB; y0 < y_end; y0 += kSB) {
+        const bool lead = y0 < y_begin;
+        const int rows = lead ? kHalo : kSB, first = lead ? y_begin - kR : y0 + kR;
+        if (!lead) before(y0 + ty * kSVR);
+        float4 v0[2], v1[2], v2[2];
+#pragma unroll
+        for (int part = 0; part < 2; ++part) {
+            const int i = threadIdx.x + 256 * part, r = i / (kSC / 4), c = (i - r * (kSC / 4)) * 4;
+            const int lx = x0 + c, ly = first + r;
+            v0[part] = v1[part] = v2[part] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (r < rows && ly >= 0 && ly < H) {
+                const long long o = (long long)ly * W;
+                v0[part] = load4<VEC>(dmu + o, lx, W);
+                v1[part] = load4<VEC>(dexx + o, lx, W);
+                v2[part] = load4<VEC>(dexy + o, lx, W);
+            }
+        }
+#pragma unroll
+        for (int part = 0; part < 2; ++part) {
+            const int i = threadIdx.x + 256 * part, r = i / (kSC / 4), c = (i - r * (kSC / 4)) * 4;
+            if (r >= rows) break;
+            float4 *d = reinterpret_cast<float4 *>(&sm.a[r][c]);
+            d[0] = make_float4(v0[part].x, v1[part].x, v0[part].y, v1[part].y);
+            d[1] = make_float4(v0[part].z, v1[part].z, v0[part].w, v1[part].w);
+            *reinterpret_cast<float4 *>(&sm.b[r][c]) = v2[part];
+        }
+        __syncthreads();
+        if (lead) {
+            if (hr < kHalo) ssim2_hfilter(sm, tp, hr, ht, hr);
+            __syncthreads();
+            continue;
+        }
+        if (y0 > y_begin) {
+            for (int i = threadIdx.x; i < kHalo * kSB; i += 256) {
+                const int r = i / kSB, c = i % kSB;
+                sm.ha[r][c] = sm.ha[kSB + r][c];
+                sm.hb[r][c] = sm.hb[kSB + r][c];
+            }
+            __syncthreads();
+        }
+        ssim2_hfilter(sm, tp, hr, ht, kHalo + hr);
+        __syncthreads();
+        float2 ga[kSVR];
+        float gb[kSVR];
+#pragma unroll
+        for (int j = 0; j < kSVR; ++j) {
+            ga[j] = make_float2(0.f, 0.f);
+            gb[j] = 0.f;
+        }
+#pragma unroll
+        for (int k = 0; k < kSVR + 2 * kR; ++k) {
+            const float2 va = sm.ha[ty * kSVR + k][tx];
+            const float vb = sm.hb[ty * kSVR + k][tx];
+#pragma unroll
+            for (int j = 0; j < kSVR; ++j) {
+                if (k - j >= 0 && k - j <= 2 * kR) {
+                    ga[j] = fp2::fma(fp2::splat(tp.w[k - j]), va, ga[j]);
+                    gb[j] = fmaf(tp.w[k - j], vb, gb[j]);
+                }
+            }
+        }
+        after(y0 + ty * kSVR, ga, gb);
+    }
+}
+
+// the images at a thread's outputs, asked for before pass 2 waits for its inputs (on tiles, 8 views of 1200 x 680:
+// 235 us with these loads after the filter, 173 us before it)
 __device__ __forceinline__ void load_outputs(const float *x, const float *y, int W, int H, int gx, int gy0,
                                              float (&px)[kSVR], float (&py)[kSVR]) {
 #pragma unroll
@@ -425,38 +470,59 @@ __device__ __forceinline__ void load_outputs(const float *x, const float *y, int
     }
 }
 
-// pass 1: per image plane (view * 3 + channel) = blockIdx.z, tile (bx, by); sums[0] += |x - y|, sums[1] += SSIM
+// pass 1: per image plane (view * 3 + channel) = blockIdx.z, strip blockIdx.x, rows from blockIdx.y seg;
+// sums[0] += |x - y|, sums[1] += SSIM
 template <bool VEC>
-__global__ void __launch_bounds__(256, 4) k_ssim1(int W, int H, const float *x, const float *y, SsimTaps tp,
+__global__ void __launch_bounds__(256, 4) k_ssim1(int W, int H, int seg, const float *x, const float *y, SsimTaps tp,
                                                   float inv_n, float *dmu, float *dexx, float *dexy, double *sums) {
     __shared__ Ssim1Smem sm;
     const long long off = (long long)blockIdx.z * W * H;
+    const int y_begin = blockIdx.y * seg;
     float2 s, l;
-    ssim_pass1_tile<false, VEC>(sm, W, H, x + off, y + off, 1.f, 0.f, tp, inv_n, dmu + off, dexx + off, dexy + off, s, l);
+    ssim_pass1_strip<false, VEC>(sm, W, H, x + off, y + off, 1.f, 0.f, tp, inv_n, dmu + off, dexx + off, dexy + off,
+                                 y_begin, min(H, y_begin + seg), s, l);
     block_add2(l, s, sums, sums + 1);
 }
 
 // pass 2: blur the three derivative maps and combine with the L1 gradient
 template <bool VEC>
-__global__ void __launch_bounds__(256, 4) k_ssim2(int W, int H, const float *x, const float *y, SsimTaps tp,
+__global__ void __launch_bounds__(256, 4) k_ssim2(int W, int H, int seg, const float *x, const float *y, SsimTaps tp,
                                                   const float *dmu, const float *dexx, const float *dexy, float l1_scale,
                                                   float w_ssim, float *d_rgb) {
     __shared__ Ssim2Smem sm;
     const long long off = (long long)blockIdx.z * W * H;
-    const int gx = blockIdx.x * kSB + (threadIdx.x & 31), gy0 = blockIdx.y * kSB + (threadIdx.x >> 5) * kSVR;
-    float2 ga[kSVR];
-    float gb[kSVR], px[kSVR], py[kSVR];
-    load_outputs(x + off, y + off, W, H, gx, gy0, px, py);
-    ssim_pass2_tile<VEC>(sm, W, H, dmu + off, dexx + off, dexy + off, tp, ga, gb);
-    if (gx >= W) return;
+    const int gx = blockIdx.x * kSB + (threadIdx.x & 31), y_begin = blockIdx.y * seg, y_end = min(H, y_begin + seg);
+    float px[kSVR], py[kSVR];
+    ssim_pass2_strip<VEC>(
+        sm, W, H, dmu + off, dexx + off, dexy + off, tp, y_begin, y_end,
+        [&](int gy0) { load_outputs(x + off, y + off, W, H, gx, gy0, px, py); },
+        [&](int gy0, const float2(&ga)[kSVR], const float(&gb)[kSVR]) {
 #pragma unroll
-    for (int j = 0; j < kSVR; ++j) {
-        if (gy0 + j >= H) break;
-        const long long o = off + (long long)(gy0 + j) * W + gx;
-        const float xv = px[j], yv = py[j];
-        const float gs = ga[j].x + 2.f * xv * ga[j].y + yv * gb[j];
-        d_rgb[o] = l1_scale * sgnf(xv - yv) - w_ssim * gs;
+            for (int j = 0; j < kSVR; ++j) {
+                if (gx >= W || gy0 + j >= y_end) break;
+                const float gs = ga[j].x + 2.f * px[j] * ga[j].y + py[j] * gb[j];
+                d_rgb[off + (long long)(gy0 + j) * W + gx] = l1_scale * sgnf(px[j] - py[j]) - w_ssim * gs;
+            }
+        });
+}
+
+// Rows of a strip's segment, in steps of kSB: a CTA costs its steps and about half of one more (the ten rows above,
+// the reduction), and the last of the waves of four CTAs per SM is half empty on average; the product is least at
+// 11 of 22 steps for 24 planes of 1200 x 680 (pass 1 and pass 2 together 329 us; 5 steps 347, 4 steps 355, 2 steps
+// 388), at one step for a single plane.
+static int ssim_segment(int W, int H, long long planes) {
+    const int steps = (H + kSB - 1) / kSB;
+    const double strips = (double)((W + kSB - 1) / kSB) * planes, slots = 4.0 * device_sm_count();
+    int best = 1;
+    double least = 0.0;
+    for (int n = 1; n <= steps; ++n) {
+        const double waves = (steps + n - 1) / n * strips / slots + 0.5, cost = std::max(1.0, waves) * (n + 0.5);
+        if (n == 1 || cost < least) {
+            least = cost;
+            best = n;
+        }
     }
+    return best * kSB;
 }
 
 __global__ void k_ssim_finish(double *scratch_sums, float w_l1, float w_ssim, double inv_n, double *loss) {
@@ -474,15 +540,15 @@ size_t ssim_scratch_bytes(int V, int W, int H) {
 }
 
 // both passes over grid.z planes
-static void launch_ssim(dim3 grid, int W, int H, const float *x, const float *y, const SsimTaps &taps, float inv_n,
+static void launch_ssim(dim3 grid, int seg, int W, int H, const float *x, const float *y, const SsimTaps &taps, float inv_n,
                         float *dmu, float *dexx, float *dexy, double *sums, float l1_scale, float w_ssim, float *d_rgb,
                         cudaStream_t s) {
     if (ssim_vec(W, x, y, dmu)) {
-        k_ssim1<true><<<grid, 256, 0, s>>>(W, H, x, y, taps, inv_n, dmu, dexx, dexy, sums);
-        k_ssim2<true><<<grid, 256, 0, s>>>(W, H, x, y, taps, dmu, dexx, dexy, l1_scale, w_ssim, d_rgb);
+        k_ssim1<true><<<grid, 256, 0, s>>>(W, H, seg, x, y, taps, inv_n, dmu, dexx, dexy, sums);
+        k_ssim2<true><<<grid, 256, 0, s>>>(W, H, seg, x, y, taps, dmu, dexx, dexy, l1_scale, w_ssim, d_rgb);
     } else {
-        k_ssim1<false><<<grid, 256, 0, s>>>(W, H, x, y, taps, inv_n, dmu, dexx, dexy, sums);
-        k_ssim2<false><<<grid, 256, 0, s>>>(W, H, x, y, taps, dmu, dexx, dexy, l1_scale, w_ssim, d_rgb);
+        k_ssim1<false><<<grid, 256, 0, s>>>(W, H, seg, x, y, taps, inv_n, dmu, dexx, dexy, sums);
+        k_ssim2<false><<<grid, 256, 0, s>>>(W, H, seg, x, y, taps, dmu, dexx, dexy, l1_scale, w_ssim, d_rgb);
     }
 }
 
@@ -494,9 +560,10 @@ int launch_loss_l1_ssim(int V, int W, int H, const float *rgb, const float *rgb_
     float *dmu = reinterpret_cast<float *>(static_cast<char *>(scratch) + 256);
     float *dexx = dmu + n, *dexy = dexx + n;
     if (cudaMemsetAsync(sums, 0, 2 * sizeof(double), s) != cudaSuccess) return GS_ERR_CUDA;
-    dim3 grid((W + kSB - 1) / kSB, (H + kSB - 1) / kSB, 3 * V);
+    const int seg = ssim_segment(W, H, 3LL * V);
+    dim3 grid((W + kSB - 1) / kSB, (H + seg - 1) / seg, 3 * V);
     const float inv_n = (float)(1.0 / (double)n);
-    launch_ssim(grid, W, H, rgb, rgb_t, taps, inv_n, dmu, dexx, dexy, sums, w_l1 * inv_n, w_ssim, d_rgb, s);
+    launch_ssim(grid, seg, W, H, rgb, rgb_t, taps, inv_n, dmu, dexx, dexy, sums, w_l1 * inv_n, w_ssim, d_rgb, s);
     k_ssim_finish<<<1, 1, 0, s>>>(sums, w_l1, w_ssim, 1.0 / (double)n, loss);
     count_launches(3);
     return check_launch();
@@ -548,10 +615,11 @@ int launch_loss_l1_ssim_noalloc(int V, int W, int H, const float *rgb, const flo
     float *dexx = dmu + plane, *dexy = dexx + plane;
     if (cudaMemsetAsync(sums, 0, 2 * sizeof(double), s) != cudaSuccess) return GS_ERR_CUDA;
     const float inv_n = (float)(1.0 / (double)n);
-    dim3 grid((W + kSB - 1) / kSB, (H + kSB - 1) / kSB, 1);
+    const int seg = ssim_segment(W, H, 1);
+    dim3 grid((W + kSB - 1) / kSB, (H + seg - 1) / seg, 1);
     for (long long p = 0; p < 3LL * V; ++p) {
         const long long off = p * plane;
-        launch_ssim(grid, W, H, rgb + off, rgb_t + off, taps, inv_n, dmu, dexx, dexy, sums, w_l1 * inv_n, w_ssim,
+        launch_ssim(grid, seg, W, H, rgb + off, rgb_t + off, taps, inv_n, dmu, dexx, dexy, sums, w_l1 * inv_n, w_ssim,
                     d_rgb + off, s);
     }
     k_ssim_finish<<<1, 1, 0, s>>>(sums, w_l1, w_ssim, 1.0 / (double)n, loss);
@@ -801,45 +869,49 @@ __global__ void __launch_bounds__(256) k_refine_depth(RefineArgs a) {
 }
 
 template <bool VEC>
-__global__ void __launch_bounds__(256, 4) k_refine_ssim1(RefineArgs a, SsimTaps tp, float inv_n) {
+__global__ void __launch_bounds__(256, 4) k_refine_ssim1(RefineArgs a, int seg, SsimTaps tp, float inv_n) {
     __shared__ Ssim1Smem sm;
     const long long plane = blockIdx.z;
     const int v = (int)(plane / 3);
     const float ea = spec_expf(a.expo[2 * v]), eb = a.expo[2 * v + 1];
     const long long off = plane * (long long)a.W * a.H;
     float2 s, l;
-    ssim_pass1_tile<true, VEC>(sm, a.W, a.H, a.rgb + off, a.rgb_t + off, ea, eb, tp, inv_n, a.dmu + off, a.dexx + off,
-                          a.dexy + off, s, l);
+    const int y_begin = blockIdx.y * seg;
+    ssim_pass1_strip<true, VEC>(sm, a.W, a.H, a.rgb + off, a.rgb_t + off, ea, eb, tp, inv_n, a.dmu + off, a.dexx + off,
+                                a.dexy + off, y_begin, min(a.H, y_begin + seg), s, l);
     block_add2(l, s, a.sums, a.sums + 1);
 }
 
 template <bool VEC>
-__global__ void __launch_bounds__(256, 4) k_refine_ssim2(RefineArgs a, SsimTaps tp, float l1_scale) {
+__global__ void __launch_bounds__(256, 4) k_refine_ssim2(RefineArgs a, int seg, SsimTaps tp, float l1_scale) {
     __shared__ Ssim2Smem sm;
     const int W = a.W, H = a.H;
     const long long plane = blockIdx.z;
     const int v = (int)(plane / 3);
     const float ea = spec_expf(a.expo[2 * v]), eb = a.expo[2 * v + 1];
     const long long off = plane * (long long)W * H;
-    float2 ba[kSVR];
-    float bb[kSVR];
-    const int gx = blockIdx.x * kSB + (threadIdx.x & 31), gy0 = blockIdx.y * kSB + (threadIdx.x >> 5) * kSVR;
+    const int gx = blockIdx.x * kSB + (threadIdx.x & 31), y_begin = blockIdx.y * seg, y_end = min(H, y_begin + seg);
     float px[kSVR], py[kSVR];
-    load_outputs(a.rgb + off, a.rgb_t + off, W, H, gx, gy0, px, py);
-    ssim_pass2_tile<VEC>(sm, W, H, a.dmu + off, a.dexx + off, a.dexy + off, tp, ba, bb);
-    float ga = 0.f, gb = 0.f;
+    float2 sa = make_float2(0.f, 0.f), sb = sa;
+    ssim_pass2_strip<VEC>(
+        sm, W, H, a.dmu + off, a.dexx + off, a.dexy + off, tp, y_begin, y_end,
+        [&](int gy0) { load_outputs(a.rgb + off, a.rgb_t + off, W, H, gx, gy0, px, py); },
+        [&](int gy0, const float2(&ba)[kSVR], const float(&bb)[kSVR]) {
+            float ga = 0.f, gb = 0.f;
 #pragma unroll
-    for (int j = 0; j < kSVR; ++j) {
-        if (gx >= W || gy0 + j >= H) continue;
-        const long long o = off + (long long)(gy0 + j) * W + gx;
-        const float xv = px[j], yv = py[j];
-        const float xt = fp::add(fp::mul(ea, xv), eb);       // I~ exactly as the FP32 L1 sign decision takes it
-        const float g = l1_scale * sgnf(xt - yv) - a.w_ssim * (ba[j].x + 2.f * xt * ba[j].y + yv * bb[j]);
-        a.d_rgb[o] = ea * g;                                 // dL/dI^ = e^a dL/dI~
-        ga += g * ea * xv;
-        gb += g;
-    }
-    block_add2(make_float2(ga, 0.f), make_float2(gb, 0.f), a.sums + 3 + v, a.sums + 3 + a.V + v);
+            for (int j = 0; j < kSVR; ++j) {
+                if (gx >= W || gy0 + j >= y_end) break;
+                const float xv = px[j], yv = py[j];
+                const float xt = fp::add(fp::mul(ea, xv), eb);   // I~ exactly as the FP32 L1 sign decision takes it
+                const float g = l1_scale * sgnf(xt - yv) - a.w_ssim * (ba[j].x + 2.f * xt * ba[j].y + yv * bb[j]);
+                a.d_rgb[off + (long long)(gy0 + j) * W + gx] = ea * g;   // dL/dI^ = e^a dL/dI~
+                ga += g * ea * xv;
+                gb += g;
+            }
+            add_to_pair(sa, ga);
+            add_to_pair(sb, gb);
+        });
+    block_add2(sa, sb, a.sums + 3 + v, a.sums + 3 + a.V + v);
 }
 
 __global__ void k_refine_finish(RefineArgs a, double inv_n) {
@@ -881,13 +953,14 @@ int launch_loss_refine(int V, int W, int H, const float *rgb, const float *rgb_t
     const int g1 = (int)std::max<long long>(1, std::min<long long>((total + 255) / 256, (long long)device_sm_count() * 8));
     const bool use_depth = a.depth && a.d_depth;
     if (use_depth) k_refine_depth<<<g1, 256, 0, s>>>(a);
-    dim3 grid((W + kSB - 1) / kSB, (H + kSB - 1) / kSB, 3 * V);
+    const int seg = ssim_segment(W, H, 3LL * V);
+    dim3 grid((W + kSB - 1) / kSB, (H + seg - 1) / seg, 3 * V);
     if (ssim_vec(W, rgb, rgb_t, a.dmu)) {
-        k_refine_ssim1<true><<<grid, 256, 0, s>>>(a, taps, inv_n);
-        k_refine_ssim2<true><<<grid, 256, 0, s>>>(a, taps, w_l1 * inv_n);
+        k_refine_ssim1<true><<<grid, 256, 0, s>>>(a, seg, taps, inv_n);
+        k_refine_ssim2<true><<<grid, 256, 0, s>>>(a, seg, taps, w_l1 * inv_n);
     } else {
-        k_refine_ssim1<false><<<grid, 256, 0, s>>>(a, taps, inv_n);
-        k_refine_ssim2<false><<<grid, 256, 0, s>>>(a, taps, w_l1 * inv_n);
+        k_refine_ssim1<false><<<grid, 256, 0, s>>>(a, seg, taps, inv_n);
+        k_refine_ssim2<false><<<grid, 256, 0, s>>>(a, seg, taps, w_l1 * inv_n);
     }
     k_refine_finish<<<1, ((V + 31) / 32) * 32, 0, s>>>(a, 1.0 / (double)n);
     count_launches(3 + use_depth);
