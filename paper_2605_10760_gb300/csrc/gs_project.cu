@@ -54,14 +54,21 @@ __device__ __forceinline__ bool may_be_visible(const float *R, const float *t, f
 // pair's position in the chunk, flagged kSlotHole for a hole (slane).  Slots beyond the capacity
 // record GS_ERR_CAPACITY for a visible pair and drop it.
 constexpr int kProjThreads = 64;
-constexpr int kProjPre = kChunk / kProjThreads;   // pairs pre-tested per thread
+constexpr int kProjWide = 256;
+// Up to two chunks per SM a block has kProjWide threads, so that a chunk is one round of the pre-test and one of
+// the chain: with room for all of them at once, a chunk's time is a chain of latencies (10 k Gaussians, 40 chunks:
+// 10.0 us with 64 threads, 5.3 us with 256; the adjoint 11.8 us and 5.3 us).  With more chunks the narrow blocks
+// are all resident and their tails, a round of few candidates, waste less.
+static bool proj_wide(const Layout &L) { return (long long)L.max_chunks * L.V <= 2LL * device_sm_count(); }
 
-__global__ void __launch_bounds__(kProjThreads) k_project(ProjArgs a) {
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS) k_project(ProjArgs a) {
+    constexpr int kProjPre = kChunk / THREADS;   // pairs pre-tested per thread
     const int v = blockIdx.y;
     __shared__ ViewEntry s_ve;
     __shared__ float s_cam[19];   // R, t, fx, fy, cx, cy, the clamp limits, then wb2
     __shared__ uint8_t s_cl[kChunk];
-    __shared__ uint32_t s_wcnt[kProjPre][kProjThreads / 32];
+    __shared__ uint32_t s_wcnt[kProjPre > 2 ? kProjPre : 2][THREADS / 32];
     __shared__ unsigned long long s_base;
     if (threadIdx.x == 0) s_ve = a.views[v];
     if (threadIdx.x < 16) s_cam[threadIdx.x] = reinterpret_cast<const float *>(a.cams + v)[threadIdx.x];
@@ -80,11 +87,11 @@ __global__ void __launch_bounds__(kProjThreads) k_project(ProjArgs a) {
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long base_i = (long long)blockIdx.x * kChunk;
-    // phase 1: pairs base_i + k kProjThreads + thread
+    // phase 1: pairs base_i + k THREADS + thread
     unsigned cmask[kProjPre];
 #pragma unroll
     for (int k = 0; k < kProjPre; ++k) {
-        const int li = k * kProjThreads + threadIdx.x;
+        const int li = k * THREADS + threadIdx.x;
         const long long i = base_i + li;
         const bool in = i < s_ve.count;
         const long long f = s_ve.pair_off + (in ? i : 0);
@@ -108,9 +115,9 @@ __global__ void __launch_bounds__(kProjThreads) k_project(ProjArgs a) {
     for (int k = 0; k < kProjPre; ++k) {
         uint32_t pre = ncand + (uint32_t)__popc(cmask[k] & lanemask_lt());
         for (int w = 0; w < warp; ++w) pre += s_wcnt[k][w];
-        if ((cmask[k] >> lane) & 1u) s_cl[pre] = (uint8_t)(k * kProjThreads + threadIdx.x);
+        if ((cmask[k] >> lane) & 1u) s_cl[pre] = (uint8_t)(k * THREADS + threadIdx.x);
 #pragma unroll
-        for (int w = 0; w < kProjThreads / 32; ++w) ncand += s_wcnt[k][w];
+        for (int w = 0; w < THREADS / 32; ++w) ncand += s_wcnt[k][w];
     }
     __syncthreads();   // s_cl complete
     // the candidates' slots: one atomic, whose result is needed only after the first round's chain.
@@ -125,11 +132,11 @@ __global__ void __launch_bounds__(kProjThreads) k_project(ProjArgs a) {
             a.st->slot_ctr = 0ull;
         }
     }
-    // phase 2: candidates r kProjThreads + thread through the decision chain
+    // phase 2: candidates r THREADS + thread through the decision chain
     uint32_t keys = 0, nvis = 0;  // touched tiles and visible pairs of this thread
-    const int rounds = (int)((ncand + kProjThreads - 1) / kProjThreads);
+    const int rounds = (int)((ncand + THREADS - 1) / THREADS);
     for (int r = 0; r < rounds; ++r) {
-        const int t = r * kProjThreads + threadIdx.x;
+        const int t = r * THREADS + threadIdx.x;
         const bool act = (uint32_t)t < ncand;
         const int li = act ? (int)s_cl[t] : 0;
         const long long i = base_i + li;
@@ -186,7 +193,6 @@ __global__ void __launch_bounds__(kProjThreads) k_project(ProjArgs a) {
     }
     keys = __reduce_add_sync(0xffffffffu, keys);   // (s_wcnt was last read before the barrier above)
     nvis = __reduce_add_sync(0xffffffffu, nvis);
-    static_assert(kProjPre >= 2, "two rows of s_wcnt");
     if (lane == 0) {
         s_wcnt[0][warp] = keys;
         s_wcnt[1][warp] = nvis;
@@ -195,7 +201,7 @@ __global__ void __launch_bounds__(kProjThreads) k_project(ProjArgs a) {
     if (threadIdx.x == 0) {
         const long long ch = s_ve.chunk_off + blockIdx.x;
         uint32_t total = 0, vis = 0;
-        for (int w = 0; w < kProjThreads / 32; ++w) {
+        for (int w = 0; w < THREADS / 32; ++w) {
             total += s_wcnt[0][w];
             vis += s_wcnt[1][w];
         }
@@ -206,7 +212,10 @@ __global__ void __launch_bounds__(kProjThreads) k_project(ProjArgs a) {
 
 void launch_project(const Layout &L, const ProjArgs &a, cudaStream_t s) {
     dim3 grid((unsigned)L.max_chunks, (unsigned)L.V);
-    k_project<<<grid, kProjThreads, 0, s>>>(a);
+    if (proj_wide(L))
+        k_project<kProjWide><<<grid, kProjWide, 0, s>>>(a);
+    else
+        k_project<kProjThreads><<<grid, kProjThreads, 0, s>>>(a);
     count_launches(1);
 }
 
@@ -228,11 +237,12 @@ constexpr int kProjBwdThreads = 64;
 
 // 16 CTAs per SM (64 registers, a small spill), so that a single view's 1954 chunks are resident
 // at once: measured faster than 10 per SM at 92 registers without spills
-__global__ void __launch_bounds__(kProjBwdThreads, 16) k_project_bwd(ProjBwdArgs a) {
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS > 64 ? 2 : 16) k_project_bwd(ProjBwdArgs a) {
     const int v = blockIdx.y;
     __shared__ ViewEntry s_ve;
     __shared__ float s_cam[18];
-    __shared__ float s_red[kProjBwdThreads / 32][6];
+    __shared__ float s_red[THREADS / 32][6];
     __shared__ uint4 s_blk;
     if (threadIdx.x == 0) s_ve = a.views[v];
     if (threadIdx.x < 16) s_cam[threadIdx.x] = reinterpret_cast<const float *>(a.cams + v)[threadIdx.x];
@@ -252,7 +262,7 @@ __global__ void __launch_bounds__(kProjBwdThreads, 16) k_project_bwd(ProjBwdArgs
     const unsigned long long b0 = s_blk.x;
     const unsigned long long n0 = b0 < vc ? min((unsigned long long)blk_candidates(s_blk.y), vc - b0) : 0ull;
     float pose[6] = {0, 0, 0, 0, 0, 0};
-    for (unsigned long long u = threadIdx.x; u < n0; u += kProjBwdThreads) {
+    for (unsigned long long u = threadIdx.x; u < n0; u += THREADS) {
         const uint32_t sl = (uint32_t)(b0 + u);
         const uint32_t lanev = a.slane[sl];
         if (lanev & kSlotHole) continue;
@@ -400,14 +410,17 @@ __global__ void __launch_bounds__(kProjBwdThreads, 16) k_project_bwd(ProjBwdArgs
     if (threadIdx.x < 6 && ch < a.chunks) {
         float r = 0.f;
 #pragma unroll
-        for (int wi = 0; wi < kProjBwdThreads / 32; ++wi) r += s_red[wi][threadIdx.x];
+        for (int wi = 0; wi < THREADS / 32; ++wi) r += s_red[wi][threadIdx.x];
         a.pose_part[(s_ve.chunk_off + blockIdx.x) * 8 + threadIdx.x] = r;
     }
 }
 
 void launch_project_bwd(const Layout &L, const ProjBwdArgs &a, cudaStream_t s) {
     dim3 grid((unsigned)L.max_chunks, (unsigned)L.V);
-    k_project_bwd<<<grid, kProjBwdThreads, 0, s>>>(a);
+    if (proj_wide(L))
+        k_project_bwd<kProjWide><<<grid, kProjWide, 0, s>>>(a);
+    else
+        k_project_bwd<kProjBwdThreads><<<grid, kProjBwdThreads, 0, s>>>(a);
     count_launches(1);
 }
 
