@@ -60,12 +60,15 @@ __device__ __forceinline__ unsigned long long vox_key(int ix, int iy, int iz) {
 // them a sector), whose number is a hash of the block: a ray of 70 voxels touches about 30 lines and its
 // neighbours in the warp the same ones, where a hash of the voxel itself touches 70 sectors of its own.  The
 // place within the line is the voxel's place in its block, XORed with hash bits (so that flat sets, which use
-// half of every block's voxels, still use all slots alike).  The sequence visits that place in the following
-// lines, then the next place in every line: the slots of one place behave like a linearly probed table of
-// random keys, and every slot is visited once in `capacity` probes.
+// half of every block's voxels, still use all slots alike).  The sequence visits that place in other lines, a
+// hashed odd number of lines apart (the lines are a power of two), then the next place in every line, so that
+// every slot is visited once in `capacity` probes: the slots of one place behave like a double-hashed table of
+// random keys.  (Carved space fills whole blocks, so a line's neighbours are no better than any other line, and
+// steps of one line would form long runs: at 89 % of the slots in use 41 probes to find a key absent, hashed
+// steps 9.  7 views into a set filled to 73 % and 89 %: 3.25 ms with steps of one line, 0.69 ms.)
 struct VoxProbe {
     unsigned long long key;
-    uint32_t block, pos, first;
+    uint32_t mix, block, pos;
 
     __device__ __forceinline__ VoxProbe(const VoxSet &s, unsigned long long k) : key(k) {
         const uint32_t lo = (uint32_t)k, hi = (uint32_t)(k >> 32);   // y's low 11 bits and z; x and y's high 10 bits
@@ -73,16 +76,17 @@ struct VoxProbe {
         // whose halves are folded onto each other, and the high part of another one
         const uint32_t h = (lo & ~0x00200001u) * 0x9e3779b1u + (hi & ~0x00000c00u) * 0x85ebca77u;
         const unsigned long long m = (unsigned long long)h * 0xc2b2ae3du;
-        const uint32_t f = (uint32_t)m ^ (uint32_t)(m >> 32);
-        block = first = __umulhi(f * 0x27d4eb2fu, s.blocks + 1u);
+        mix = (uint32_t)m ^ (uint32_t)(m >> 32);
+        block = home(s);
         const uint32_t place = ((hi >> 10) & 3u) | ((lo >> 19) & 4u) | ((lo << 3) & 8u);
-        pos = (place ^ f) & s.pos;
+        pos = (place ^ mix) & s.pos;
     }
+    __device__ __forceinline__ uint32_t home(const VoxSet &s) const { return __umulhi(mix * 0x27d4eb2fu, s.blocks + 1u); }
     __device__ __forceinline__ size_t slot(const VoxSet &s) const { return ((size_t)block << s.shift) | pos; }
     // the next slot; false once all have been visited (`places` counts the places done)
     __device__ __forceinline__ bool next(const VoxSet &s, uint32_t &places) {
-        block = (block + 1u) & s.blocks;
-        if (block == first) {
+        block = (block + ((mix >> 5) | 1u)) & s.blocks;
+        if (block == home(s)) {
             pos = (pos + 1u) & s.pos;
             return ++places <= s.pos;
         }
@@ -101,7 +105,8 @@ __device__ __forceinline__ bool voxset_insert(const VoxSet &s, unsigned long lon
             const unsigned long long prev = atomicCAS(slot, kEmptyKey, p.key);
             if (prev == kEmptyKey || prev == p.key) return true;
         }
-    } while (p.next(s, places));
+        // a set that was found full stays full: one place of every line is enough to give up again
+    } while (p.next(s, places) && (places == 0u || *(volatile int32_t *)s.status != GS_ERR_CAPACITY));
     atomicCAS(s.status, 0, GS_ERR_CAPACITY);
     return false;
 }

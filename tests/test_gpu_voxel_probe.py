@@ -61,3 +61,20 @@ def test_boxes_of_uneven_sizes(n):
     s = R.VoxSet(1 << 20)
     s.add_boxes(means, logs, 1.0, V)
     assert s.status() == (0, len(want)) and s.keys() == want
+
+
+def test_an_overfull_set_reports_and_keeps_its_capacity():
+    from paper_2605_10760_gb300 import _lib as L, raster as R
+    cap = 1 << 12
+    means, keys = _centres("scattered", 4 * cap, np.random.default_rng(1))
+    small = torch.full((4 * cap, 3), -12.0, device="cuda")
+    s = R.VoxSet(cap)
+    for _ in range(2):
+        s.add_boxes(means, small, 3.0, V)
+        assert s.status() == (L.GS_ERR_CAPACITY, cap)
+    assert s.keys() < keys
+    keep = R.dedup_keep(means, s, None, V)
+    assert int((keep == 0).sum()) == cap
+    s.clear()
+    s.add_boxes(means[:cap], small[:cap], 3.0, V)
+    assert s.status() == (0, cap)
