@@ -674,7 +674,7 @@ def fusion_bench(R, S, torch, voxel=0.05, k=3.0, stride=2, reps=3):
                                           "voxel (random DRAM sectors)"},
                          "occupied_gaussians_per_s": tgt.n / (ms["occupied"] * 1e-3),
                          "free_rays_per_s": rays / (ms["free"] * 1e-3),
-                         "note": "hash insertion (occupied, free) is bound by L2 compare-and-swap traffic"}}
+                         "note": "hash insertion (occupied, free) is bound by instruction issue"}}
 
 
 def fused_map(R, S, torch, steps=3):
@@ -889,7 +889,7 @@ def main():
     fp32_peak = 152 * 128 * 2 * peaks["sm_max_mhz"] * 1e6 / 1e12   # TFLOP/s at max SM clock
     # DRAM bytes (read + write) of one launch from an ncu capture of this workload's current
     # kernel code (profiles/*_room500k.md); a stage without such a capture reports None
-    traffic = {"render_fwd_l1": 26_724_352, "render_bwd": 35_204_864}
+    traffic = {"render_fwd_l1": 27_051_264, "render_bwd": 33_723_904}
     if dom in ("render_fwd_l1", "render_bwd"):
         flops = stats["fwd_pairs"] * FLOP_FWD if dom == "render_fwd_l1" else stats["bwd_pairs"] * FLOP_BWD
         ach = flops / (stage_ms[dom] * 1e-3) / 1e12
