@@ -200,8 +200,9 @@ struct RayArgs {
 // Bound by the instructions of a step (about 40: the analyser, the hash, the probe), not by memory: the rays of a
 // patch walk together through the lines near the camera.  8 views of 600 x 340 rays, some 70 voxels each, a set of
 // 2^25: 442 us (419 us with probe steps of one line, see VoxProbe; 48 warps an SM 477 us); before those hashed steps
-// 467 us with a warp's rays along a row; 827 us with voxels hashed one by one and 64-bit indices.  Settling a voxel only after the next one's load was issued: 650 us (more instructions,
-// and more slots found empty that another warp had just filled).
+// 467 us with a warp's rays along a row; 827 us with voxels hashed one by one and 64-bit indices.  Settling a voxel
+// only after the next one's load was issued: 650 us (more instructions, and more slots found empty that another
+// warp had just filled).
 __global__ void __launch_bounds__(256, 8) k_add_rays(RayArgs a) {
     const long long total = (long long)a.V * a.pw * a.ph * 32;
     for (long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x; r < total; r += (long long)gridDim.x * blockDim.x) {
