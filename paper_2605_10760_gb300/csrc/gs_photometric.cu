@@ -26,7 +26,7 @@
 namespace gs {
 
 constexpr int kPhoThreads = 256;
-constexpr int kPhoPPT = 2;            // anchor pixels per thread per step
+constexpr int kPhoPPT = 2;            // anchor pixels per thread per step: the halves of the packed chain
 constexpr int kPhoSums = 37;          // S (28, upper triangle row-major), s_g (7), cost, count
 constexpr int kPhoStride = 40;        // doubles per partial
 
@@ -50,12 +50,16 @@ __device__ void pho_quat_matrix(const float *qin, float *M) {
     M[8] = sub(1.0f, mul(2.0f, add(mul(x, x), mul(y, y))));
 }
 
+// The rounded product a b as a b - 0 (nz: -0 in both halves, read at run time): the assembler joins a packed
+// product and a following packed sum into one fused operation, which the chain must not have.
+__device__ __forceinline__ float2 mul2(float2 a, float2 b, float2 nz) { return fp2::fma(a, b, nz); }
+
 // (M v)_i = (M_i0 v_0 + M_i1 v_1) + M_i2 v_2 and the transposed form, every operation rounded.
-__device__ __forceinline__ float pho_row(const float *M, int i, float a, float b, float c) {
-    return fp::add(fp::add(fp::mul(M[3 * i], a), fp::mul(M[3 * i + 1], b)), fp::mul(M[3 * i + 2], c));
+__device__ __forceinline__ float2 pho_row(const float2 *M, int i, float2 a, float2 b, float2 c, float2 nz) {
+    return fp2::add(fp2::add(mul2(M[3 * i], a, nz), mul2(M[3 * i + 1], b, nz)), mul2(M[3 * i + 2], c, nz));
 }
-__device__ __forceinline__ float pho_col(const float *M, int i, float a, float b, float c) {
-    return fp::add(fp::add(fp::mul(M[i], a), fp::mul(M[3 + i], b)), fp::mul(M[6 + i], c));
+__device__ __forceinline__ float2 pho_col(const float2 *M, int i, float2 a, float2 b, float2 c, float2 nz) {
+    return fp2::add(fp2::add(mul2(M[i], a, nz), mul2(M[3 + i], b, nz)), mul2(M[6 + i], c, nz));
 }
 
 struct PhoEdgeConst {
@@ -115,32 +119,46 @@ struct PhoSample {
     float w0, w1, w2, c0, c1, iz;     // global point, target camera x, y and 1 / z
 };
 
-// The FP32 decision chain of one anchor pixel (column px as a float, yn of its row, depth d).
-__device__ __forceinline__ PhoSample pho_chain(const PhoEdgeConst &k, float px, float yn, float d, float near_plane,
-                                               int W, int H) {
-    using namespace fp;
+// The chain's constants as both halves of packed operands (differences add the negative).
+struct PhoPairConst {
+    float2 Rs[9], nts[3], ncx, ifx;
+    float2 Q1[9], t1[3], s1;
+    float2 Q2[9], nt2[3], is2;
+    float2 Ra[9], ta[3], Ka[4];
+    float2 nz;                        // -0 (see mul2)
+};
+
+__device__ void pho_pair_consts(const PhoEdgeConst &k, PhoPairConst &c) {
+    using fp2::splat;
+    for (int i = 0; i < 9; ++i) {
+        c.Rs[i] = splat(k.Rs[i]);
+        c.Q1[i] = splat(k.Q1[i]);
+        c.Q2[i] = splat(k.Q2[i]);
+        c.Ra[i] = splat(k.Ra[i]);
+    }
+    for (int i = 0; i < 3; ++i) {
+        c.nts[i] = splat(-k.ts[i]);
+        c.t1[i] = splat(k.t1[i]);
+        c.nt2[i] = splat(-k.t2[i]);
+        c.ta[i] = splat(k.ta[i]);
+    }
+    for (int i = 0; i < 4; ++i) c.Ka[i] = splat(k.Ka[i]);
+    c.nz = splat(-0.0f);
+    c.ncx = splat(-k.Ks[2]);
+    c.ifx = splat(k.ifx);
+    c.s1 = splat(k.s1);
+    c.is2 = splat(k.is2);
+}
+
+// One pixel's end of the chain: its decisions and its bilinear cell.
+__device__ __forceinline__ PhoSample pho_sample(float d, float near_plane, float c2, float sx, float sy, int W, int H,
+                                                float w0, float w1, float w2, float c0, float c1, float iz) {
     PhoSample o;
     o.ok = false;
     o.x0 = o.y0 = 0;
     o.ax = o.ay = o.w0 = o.w1 = o.w2 = o.c0 = o.c1 = o.iz = 0.0f;
     if (!(d > 0.0f) || !(d < __int_as_float(0x7f800000))) return o;
-    const float xn = mul(sub(add(px, 0.5f), k.Ks[2]), k.ifx);
-    const float pc0 = sub(mul(xn, d), k.ts[0]), pc1 = sub(mul(yn, d), k.ts[1]), pc2 = sub(d, k.ts[2]);
-    const float p0 = pho_col(k.Rs, 0, pc0, pc1, pc2), p1 = pho_col(k.Rs, 1, pc0, pc1, pc2),
-                p2 = pho_col(k.Rs, 2, pc0, pc1, pc2);
-    const float w0 = add(mul(k.s1, pho_row(k.Q1, 0, p0, p1, p2)), k.t1[0]);
-    const float w1 = add(mul(k.s1, pho_row(k.Q1, 1, p0, p1, p2)), k.t1[1]);
-    const float w2 = add(mul(k.s1, pho_row(k.Q1, 2, p0, p1, p2)), k.t1[2]);
-    const float d0 = sub(w0, k.t2[0]), d1 = sub(w1, k.t2[1]), d2 = sub(w2, k.t2[2]);
-    const float q0 = mul(pho_col(k.Q2, 0, d0, d1, d2), k.is2), q1 = mul(pho_col(k.Q2, 1, d0, d1, d2), k.is2),
-                q2 = mul(pho_col(k.Q2, 2, d0, d1, d2), k.is2);
-    const float c0 = add(pho_row(k.Ra, 0, q0, q1, q2), k.ta[0]);
-    const float c1 = add(pho_row(k.Ra, 1, q0, q1, q2), k.ta[1]);
-    const float c2 = add(pho_row(k.Ra, 2, q0, q1, q2), k.ta[2]);
     if (!(c2 > near_plane)) return o;
-    const float iz = div(1.0f, c2);
-    const float sx = sub(add(mul(k.Ka[0], mul(c0, iz)), k.Ka[2]), 0.5f);
-    const float sy = sub(add(mul(k.Ka[1], mul(c1, iz)), k.Ka[3]), 0.5f);
     if (!(sx >= 0.0f) || !(sx < (float)(W - 1)) || !(sy >= 0.0f) || !(sy < (float)(H - 1))) return o;
     const float fx0 = floorf(sx), fy0 = floorf(sy);
     o.ok = true;
@@ -157,12 +175,44 @@ __device__ __forceinline__ PhoSample pho_chain(const PhoEdgeConst &k, float px, 
     return o;
 }
 
+// The FP32 decision chain of two anchor pixels of a row (columns px as floats, yn of the row, depths d) as the halves
+// of packed operands, each rounded like the scalar operation (the same bits).  The sums over pixels stay one pixel
+// at a time: their order is part of the FP64 outputs.  16 edges of 1200 x 680, kernel and finish: 281 us, 322 us with
+// a scalar chain; with the sums packed too 261 us, but H, g and cost 4e-5 apart.
+__device__ __forceinline__ void pho_chain(const PhoPairConst &k, float2 px, float yn, float2 d, float near_plane, int W,
+                                          int H, PhoSample (&o)[2]) {
+    using namespace fp2;
+    const float2 xn = mul2(add(add(px, splat(0.5f)), k.ncx), k.ifx, k.nz);
+    const float2 pc0 = add(mul2(xn, d, k.nz), k.nts[0]), pc1 = add(mul2(splat(yn), d, k.nz), k.nts[1]), pc2 = add(d, k.nts[2]);
+    const float2 p0 = pho_col(k.Rs, 0, pc0, pc1, pc2, k.nz), p1 = pho_col(k.Rs, 1, pc0, pc1, pc2, k.nz),
+                 p2 = pho_col(k.Rs, 2, pc0, pc1, pc2, k.nz);
+    const float2 w0 = add(mul2(k.s1, pho_row(k.Q1, 0, p0, p1, p2, k.nz), k.nz), k.t1[0]);
+    const float2 w1 = add(mul2(k.s1, pho_row(k.Q1, 1, p0, p1, p2, k.nz), k.nz), k.t1[1]);
+    const float2 w2 = add(mul2(k.s1, pho_row(k.Q1, 2, p0, p1, p2, k.nz), k.nz), k.t1[2]);
+    const float2 d0 = add(w0, k.nt2[0]), d1 = add(w1, k.nt2[1]), d2 = add(w2, k.nt2[2]);
+    const float2 q0 = mul2(pho_col(k.Q2, 0, d0, d1, d2, k.nz), k.is2, k.nz);
+    const float2 q1 = mul2(pho_col(k.Q2, 1, d0, d1, d2, k.nz), k.is2, k.nz);
+    const float2 q2 = mul2(pho_col(k.Q2, 2, d0, d1, d2, k.nz), k.is2, k.nz);
+    const float2 c0 = add(pho_row(k.Ra, 0, q0, q1, q2, k.nz), k.ta[0]);
+    const float2 c1 = add(pho_row(k.Ra, 1, q0, q1, q2, k.nz), k.ta[1]);
+    const float2 c2 = add(pho_row(k.Ra, 2, q0, q1, q2, k.nz), k.ta[2]);
+    const float2 iz = make_float2(fp::div(1.0f, c2.x), fp::div(1.0f, c2.y));
+    const float2 sx = add(add(mul2(k.Ka[0], mul2(c0, iz, k.nz), k.nz), k.Ka[2]), splat(-0.5f));
+    const float2 sy = add(add(mul2(k.Ka[1], mul2(c1, iz, k.nz), k.nz), k.Ka[3]), splat(-0.5f));
+    o[0] = pho_sample(d.x, near_plane, c2.x, sx.x, sy.x, W, H, w0.x, w1.x, w2.x, c0.x, c1.x, iz.x);
+    o[1] = pho_sample(d.y, near_plane, c2.y, sx.y, sy.y, W, H, w0.y, w1.y, w2.y, c0.y, c1.y, iz.y);
+}
+
 __global__ void __launch_bounds__(kPhoThreads, 2) k_pho_edge(PhoArgs a) {
     using namespace fp;
     __shared__ PhoEdgeConst k;
+    __shared__ PhoPairConst kc;
     __shared__ float red[kPhoThreads / 32][kPhoSums];
     const int e = blockIdx.y;
-    if (threadIdx.x == 0) k.valid = pho_load_edge(a, e, k) ? 1 : 0;
+    if (threadIdx.x == 0) {
+        k.valid = pho_load_edge(a, e, k) ? 1 : 0;
+        if (k.valid) pho_pair_consts(k, kc);
+    }
     __syncthreads();
 
     float S[28], sg[7], cost = 0.0f, cnt = 0.0f;
@@ -194,9 +244,8 @@ __global__ void __launch_bounds__(kPhoThreads, 2) k_pho_edge(PhoArgs a) {
                 for (int ch = 0; ch < 3; ++ch) src[p][ch] = in ? __ldg(k.img_s + ch * plane + os_row + px) : 0.0f;
             }
             PhoSample sm[kPhoPPT];
-#pragma unroll
-            for (int p = 0; p < kPhoPPT; ++p)
-                sm[p] = pho_chain(k, (float)((rx0 + p * kPhoThreads) * st), yn, dd[p], a.near_plane, W, H);
+            pho_chain(kc, make_float2((float)(rx0 * st), (float)((rx0 + kPhoThreads) * st)), yn,
+                      make_float2(dd[0], dd[1]), a.near_plane, W, H, sm);
             float tap[kPhoPPT][3][4];
 #pragma unroll
             for (int p = 0; p < kPhoPPT; ++p) {
