@@ -341,6 +341,11 @@ __device__ __forceinline__ float2 spec_exp_neg(float2 s) {
 }
 constexpr float kFastCut = 80.0f;   // sigma cut-offs below it keep spec_exp_neg in range
 
+// Values that a weight of 0 takes out of a sum, alone or times one another: finite and far below overflow.
+__device__ __forceinline__ bool tame(float a, float b, float c, float d) {   // false with a NaN
+    return (fabsf(a) + fabsf(b)) + (fabsf(c) + fabsf(d)) < 1e15f;
+}
+
 // spec_sigma at two pixels of one column (dy per pixel)
 __device__ __forceinline__ float2 spec_sigma2(float A, float B, float C, float dx, float2 dy) {
     const float2 q = fp2::fma(fp2::splat(fp::mul(A, dx)), fp2::splat(dx), fp2::mul(fp2::mul(fp2::splat(C), dy), dy));

@@ -176,9 +176,10 @@ __global__ void __launch_bounds__(THREADS) k_project(ProjArgs a) {
                 cnt = (uint32_t)((o.x1 - o.x0) * (o.y1 - o.y0));
                 a.slot[f] = (uint32_t)slot;
                 float4 *rec = a.proj + 3 * slot;
-                // sigma beyond which alpha < alpha_min is certain (see gs_render.cu); +inf disables the cut
+                // sigma beyond which alpha < alpha_min is certain (see gs_render.cu); +inf disables the cut, also
+                // for a colour or depth that only the compositing's SLOW walk keeps to the pixels blending it
                 float cut = __int_as_float(0x7f800000);
-                if (a.alpha_min > 0.0f) {
+                if (a.alpha_min > 0.0f && tame(c0, c1, c2, o.z)) {
                     if (op > 0.0f) cut = logf(op / a.alpha_min) + 1e-3f;
                     else if (op <= 0.0f) cut = -1.0f;
                 }
