@@ -317,6 +317,8 @@ __device__ __forceinline__ void add_to_pair(float2 &s, float x) {
     s.y = fp::add(s.y, fp::add(fp::sub(s.x, fp::sub(t, b)), fp::sub(x, b)));
     s.x = t;
 }
+// the sum (the second float of an infinite one is NaN: infinity minus infinity)
+__device__ __forceinline__ double pair_value(float2 s) { return isinf(s.x) ? (double)s.x : (double)s.x + s.y; }
 
 // spec_expf2(-s) for components s in [0, 80], bit for bit.  Everything runs on s and -r with the signs of
 // the odd coefficients turned (rounding to nearest is symmetric), so nothing is negated; no range is

@@ -197,7 +197,7 @@ __device__ __forceinline__ void block_add2(float2 a, float2 b, double *pa, doubl
         add_to_pair(b, bx);
     }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) s_part[warp] = make_double2((double)a.x + a.y, (double)b.x + b.y);
+    if (lane == 0) s_part[warp] = make_double2(pair_value(a), pair_value(b));
     __syncthreads();
     if (threadIdx.x < 2) {
         double v = 0.0;
@@ -875,7 +875,7 @@ __global__ void __launch_bounds__(256) k_refine_depth(RefineArgs a) {
         }
         store_vec(a.d_depth + i, g);
     }
-    block_add_double((double)acc.x + acc.y, a.sums + 2);
+    block_add_double(pair_value(acc), a.sums + 2);
 }
 
 template <bool VEC>

@@ -510,7 +510,7 @@ __global__ void __launch_bounds__(TW *TH / kPPT, kResident<TW, TH, NB>) k_render
     for (int o = 16; o > 0; o >>= 1) pairs += __shfl_xor_sync(0xffffffffu, pairs, o);
     if ((tid & 31) == 0 && pairs) atomicAdd(&a.st->fwd_pairs, pairs);
     if (a.rgb_t) {   // one double atomic per warp for the loss
-        double l = ((double)l1_rgb.x + l1_rgb.y) * a.sc_rgb + ((double)l1_d.x + l1_d.y) * a.sc_d;
+        double l = pair_value(l1_rgb) * a.sc_rgb + pair_value(l1_d) * a.sc_d;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
         if ((tid & 31) == 0 && l != 0.0) atomicAdd(a.loss, l);
