@@ -122,6 +122,7 @@ int compute_layout(const gs_problem *pb, Layout *L) {
     // scan_state .. ranges before the radix binning
     L->o_tcnt = o; o = align256(o + sizeof(uint32_t) * (size_t)L->G);
     L->o_tscan = o; o = align256(o + sizeof(unsigned long long) * (size_t)((L->G + kScanTile - 1) / kScanTile));
+    L->o_coop = o; o = align256(o + sizeof(uint32_t) * kCoopWords);
     L->o_scan_state = o; o = align256(o + sizeof(unsigned long long) * L->scan_parts);
     L->o_vscan = o; o = align256(o + sizeof(unsigned long long) * L->scan_parts);
     const long long emit_pairs = std::max<long long>(1, std::min(L->cap, P));
@@ -424,6 +425,7 @@ static BinArgs make_bin_args(const Layout &L, void *ws) {
     a.chunks = L.chunks_total;
     a.tile_cnt = ws_ptr<uint32_t>(ws, L.o_tcnt);
     a.tile_scan_state = ws_ptr<unsigned long long>(ws, L.o_tscan);
+    a.coop = ws_ptr<uint32_t>(ws, L.o_coop);
     a.items = ws_ptr<uint4>(ws, L.o_srec);
     a.words = ws_ptr<unsigned long long>(ws, L.o_keys[(L.passes & 1) ^ 1]);
     a.extra = ws_ptr<uint2>(ws, L.o_extra);

@@ -354,6 +354,20 @@ __device__ __forceinline__ int merge_split(At at, int a0, int na, int b0, int nb
     return lo;
 }
 
+// The same for runs of na and nb words at r, by a warp: 32 probes a step, so that runs in global memory cost a few
+// loads in a chain instead of one per bit of their length.
+__device__ __forceinline__ int warp_split(const word_t *r, int na, int nb, int d, int lane) {
+    int lo = max(0, d - nb), hi = min(d, na);
+    while (lo < hi) {                     // (lo and hi are the same in every lane)
+        const int step = (hi - lo + 31) >> 5, mid = lo + (lane + 1) * step - 1;
+        const int below = __popc(__ballot_sync(0xffffffffu, mid < hi && r[mid] < r[na + d - 1 - mid]));
+        const int from = lo + below * step;
+        hi = min(hi, from + step - 1);
+        lo = from;
+    }
+    return lo;
+}
+
 // KPT outputs of the merge of A and B in shared memory from diagonal d on (past the end: ~0)
 template <int KPT>
 __device__ __forceinline__ void merge_regs(const word_t *s, int a0, int na, int b0, int nb, int d, word_t (&out)[KPT]) {
@@ -555,9 +569,205 @@ __device__ __forceinline__ void sort_short(const BinArgs &a, long long g, uint32
     else warp_list<8>(a, kout, vout, g, r.x, n, slots, lane);
 }
 
-// The first a.long_blocks CTAs take the longer lists (a CTA each, longest first): runs of 8 words per
-// thread sorted in shared memory, the runs of a longer list merged pairwise, a run of outputs at a time,
-// between the tile's slices of the two key buffers.  The other CTAs sort the short lists beside them, a
+// Output block b (kRun words) of one merge level of a list of n words: runs of w words of `in` merged pairwise into
+// `out`; whole CTA.  Two warps find where the block's first and last outputs split the two runs.
+template <int THREADS>
+__device__ __forceinline__ void merge_block(word_t *s, int *split, const word_t *in, word_t *out, int n, int b, long long w) {
+    constexpr int kRun = kTlKPT * THREADS;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int base = (int)((long long)b * kRun / (2 * w) * (2 * w));
+    const int na = (int)min(w, (long long)n - base), nb = (int)min(w, (long long)n - base - na);
+    const int d0 = b * kRun - base, d1 = min(d0 + kRun, na + nb);
+    if (warp < 2) {
+        const int at = warp_split(in + base, na, nb, warp ? d1 : d0, lane);
+        if (lane == 0) split[warp] = at;
+    }
+    __syncthreads();
+    const int a0 = split[0], ca = split[1] - a0, cb = d1 - d0 - ca;
+    const word_t *ra = in + base + a0, *rb = in + base + na + (d0 - a0);
+    for (int e = tid; e < ca + cb; e += THREADS) s[pd(e)] = e < ca ? ra[e] : rb[e - ca];
+    __syncthreads();
+    word_t x[kTlKPT];
+    const bool act = tid * kTlKPT < ca + cb;
+    if (act) merge_regs<kTlKPT>(s, 0, ca, ca, cb, tid * kTlKPT, x);
+    __syncthreads();
+    if (act) {
+#pragma unroll
+        for (int r = 0; r < kTlKPT; ++r) s[pd(tid * kTlKPT + r)] = x[r];
+    }
+    __syncthreads();
+    for (int e = tid; e < ca + cb; e += THREADS) out[b * kRun + e] = s[pd(e)];
+    __syncthreads();
+}
+
+// Keys, values and records of `len` sorted words from position r0 of tile g's list at s0; whole CTA.  (`in` may be the
+// key buffer itself: an entry's key is written by the thread that read its word.)
+template <int THREADS>
+__device__ __forceinline__ void finish_run(const BinArgs &a, word_t *s, const word_t *in, long long g, long long s0, int r0, int len) {
+    uint32_t *slots = reinterpret_cast<uint32_t *>(s);
+    uint64_t *kout = a.keys[a.passes & 1];
+    uint32_t *vout = a.vals[a.passes & 1];
+    for (int e = threadIdx.x; e < len; e += THREADS) slots[e] = emit_entry(a, kout, vout, g, s0 + r0 + e, in[r0 + e]);
+    __syncthreads();
+    copy_records<THREADS>(a, s0 + r0, len, threadIdx.x, [&](int e) { return slots[e]; });
+    __syncthreads();
+}
+
+// Lists of more than kCoopMin words and of more than a 192nd of all keys are sorted by all long-list CTAs together: a
+// tile may hold every Gaussian of a view, and a list of 131 k words takes one CTA 3.1 ms.  The work is split into items of one run or output block each:
+// stage 0 sorts the runs in place, each further stage is one merge level, the last one writes keys, values and
+// records.  CTAs claim items by a ticket, all lists' items of a stage before the next stage's, and an item waits
+// until every item of its list's earlier stages is counted in the list's done word.  All those have smaller
+// tickets, whose holders are running CTAs that wait for smaller ones only, so no wait depends on a CTA that has yet
+// to start (and each is bounded).  The share of the keys keeps a view of many long lists at one list per CTA, without
+// waits, and bounds the number of shared lists by kCoopLists.
+//   Binning of a 640 x 480 view, us, one CTA per list / lists shared: 60 k Gaussians in 4 tiles 465 / 111, 400 k
+// 3268 / 324, 2 M 22976 / 1306 (the emission takes 190 and 960 of it); 400 k in 36 tiles 538 / 185; 2 M in 144 tiles
+// 1062 / 698.  (kCoopMin 16384: 400 k in 36 tiles 425.)  No list is shared in a 500 k room (67 and 67 us) or in 32
+// views of submaps (503 and 508).
+constexpr int kCoopLists = 192;
+constexpr uint32_t kCoopMin = 4096;
+
+struct CoopLists {
+    uint32_t start[kCoopLists], n[kCoopLists], g[kCoopLists];
+    uint32_t upto[kCoopLists];           // items of the stage in this and the lists before
+    uint32_t warp_cnt[32];
+    uint32_t ticket;
+    int count, levels, ok;
+};
+static_assert(kCoopWords == 1 + kCoopLists, "ticket and done words");
+
+__device__ __forceinline__ int merge_levels(uint32_t runs) { return runs > 1u ? 32 - __clz(runs - 1u) : 0; }
+
+// The shared lists in claim order (the same in every CTA): of the first `cand` claims those of more than `above` words.
+template <int THREADS>
+__device__ __forceinline__ void coop_collect(const BinArgs &a, CoopLists &c, const uint32_t *coff, long long cand, uint32_t above,
+                                             unsigned long long K) {
+    constexpr int kRun = kTlKPT * THREADS;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (threadIdx.x == 0) c.count = c.levels = 0;
+    __syncthreads();
+    for (long long i0 = 0; i0 < cand; i0 += THREADS) {
+        const long long i = i0 + threadIdx.x;
+        const long long g = i < cand ? claim_at(coff, a.clist, a.G, i) : a.G;
+        const uint2 r = g < a.G ? reinterpret_cast<const uint2 *>(a.ranges)[g] : make_uint2(0u, 0u);
+        const bool in = r.y > r.x && (unsigned long long)r.y <= K && r.y - r.x > above;
+        const unsigned vote = __ballot_sync(0xffffffffu, in);
+        if (lane == 0) c.warp_cnt[warp] = (uint32_t)__popc(vote);
+        __syncthreads();
+        uint32_t at = (uint32_t)c.count + (uint32_t)__popc(vote & lanemask_lt()), all = 0;
+#pragma unroll 1
+        for (int w = 0; w < THREADS / 32; ++w) {
+            if (w < warp) at += c.warp_cnt[w];
+            all += c.warp_cnt[w];
+        }
+        if (in && at < (uint32_t)kCoopLists) {
+            c.start[at] = r.x;
+            c.n[at] = r.y - r.x;
+            c.g[at] = (uint32_t)g;
+            atomicMax(&c.levels, merge_levels((r.y - r.x + kRun - 1u) / kRun));
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) c.count = min(c.count + (int)all, kCoopLists);
+        __syncthreads();
+    }
+}
+
+// upto[] of a stage and its number of items; whole CTA
+template <int THREADS>
+__device__ __forceinline__ uint32_t coop_stage(CoopLists &c, int stage) {
+    constexpr uint32_t kRun = kTlKPT * THREADS;
+    const int lane = threadIdx.x & 31;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        uint32_t before = 0;
+        for (int i0 = 0; i0 < c.count; i0 += 32) {
+            const int i = i0 + lane;
+            const uint32_t runs = i < c.count ? (c.n[i] + kRun - 1u) / kRun : 0u;
+            uint32_t x = stage == 0 || stage > c.levels || merge_levels(runs) >= stage ? runs : 0u;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += y;
+            }
+            if (i < c.count) c.upto[i] = before + x;
+            before += __shfl_sync(0xffffffffu, x, 31);
+        }
+    }
+    __syncthreads();
+    return c.upto[c.count - 1];
+}
+
+// Waits until `want` items of a list are done (thread 0; bounded).  The barrier after it makes what their CTAs wrote
+// visible to the whole CTA.
+__device__ __forceinline__ bool coop_wait(const BinArgs &a, const uint32_t *done, uint32_t want) {
+    for (unsigned long long spins = 0; ld_relaxed_u32(done) < want; ++spins) {
+        if (spins > a.spin_limit) {
+            record_error(a.st, GS_ERR_TIMEOUT, 13);
+            return false;
+        }
+        __nanosleep(64);
+    }
+    __threadfence();
+    return true;
+}
+
+// false after a wait that ran out
+template <int THREADS>
+__device__ __forceinline__ bool coop_sort(const BinArgs &a, CoopLists &c, word_t *s, int *split) {
+    constexpr int kRun = kTlKPT * THREADS;
+    const int tid = threadIdx.x, last = c.levels + 1;
+    uint64_t *kout = a.keys[a.passes & 1];
+    if (tid == 0) c.ticket = atomicAdd(a.coop, 1u);
+    uint32_t before = 0, items = coop_stage<THREADS>(c, 0);   // (its barriers publish the ticket)
+    int stage = 0;
+    for (;;) {
+        const uint32_t t = c.ticket;
+        while (stage <= last && t - before >= items) {
+            before += items;
+            if (++stage <= last) items = coop_stage<THREADS>(c, stage);
+        }
+        if (stage > last) return true;
+        const uint32_t at = t - before;
+        int lo = 0, hi = c.count - 1;     // the list: smallest i with upto[i] > at
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (c.upto[mid] > at) hi = mid;
+            else lo = mid + 1;
+        }
+        const int i = lo, b = (int)(at - (i ? c.upto[i - 1] : 0u)), n = (int)c.n[i], r0 = b * kRun;
+        const uint32_t runs = (c.n[i] + kRun - 1u) / kRun;
+        const int levels = merge_levels(runs);
+        uint32_t next = 0;
+        if (tid == 0) {
+            next = atomicAdd(a.coop, 1u);    // on its way while the item is worked on
+            c.ok = stage == 0 || coop_wait(a, a.coop + 1 + i, runs * (uint32_t)min(stage, levels + 1));
+        }
+        __syncthreads();
+        if (!c.ok) return false;
+        word_t *buf[2] = {a.words + c.start[i], reinterpret_cast<word_t *>(kout) + c.start[i]};
+        if (stage == 0) {
+            const int len = min(kRun, n - r0);
+            sort_smem<THREADS>(s, buf[0] + r0, len);
+            for (int e = tid; e < len; e += THREADS) buf[0][r0 + e] = s[pd(e)];
+        } else if (stage < last) {
+            merge_block<THREADS>(s, split, buf[(stage - 1) & 1], buf[stage & 1], n, b, (long long)kRun << (stage - 1));
+        } else {
+            finish_run<THREADS>(a, s, buf[levels & 1], c.g[i], c.start[i], r0, min(kRun, n - r0));
+        }
+        __syncthreads();
+        if (tid == 0) {
+            __threadfence();                 // the item's words before its count
+            atomicAdd(a.coop + 1 + i, 1u);
+            c.ticket = next;
+        }
+        __syncthreads();
+    }
+}
+
+// The first a.long_blocks CTAs take the longer lists (the longest of them together, then a CTA each, longest first):
+// runs of 8 words per thread sorted in shared memory, the runs of a longer list merged pairwise, a run of outputs
+// at a time, between the tile's slices of the two key buffers.  The other CTAs sort the short lists beside them, a
 // tile per warp.
 template <int kTlThreads>
 constexpr size_t kTileSortSmem = sizeof(word_t) * (kTlKPT * kTlThreads + kTlThreads);
@@ -575,7 +785,8 @@ __global__ void __launch_bounds__(kTlThreads, 1024 / kTlThreads) k_tile_sort(Bin
         return;
     }
     __shared__ uint32_t coff[kClaimClasses + 1];
-    __shared__ int s_split[kTlThreads + 1];
+    __shared__ int s_split[2];
+    __shared__ CoopLists s_coop;
     const int tid = threadIdx.x;
     uint64_t *kout = a.keys[a.passes & 1];
     uint32_t *vout = a.vals[a.passes & 1];
@@ -583,6 +794,12 @@ __global__ void __launch_bounds__(kTlThreads, 1024 / kTlThreads) k_tile_sort(Bin
     __syncthreads();
     const long long nlong = min((long long)coff[kLongClass + 1], a.G);
     const unsigned long long K = min(a.st->num_keys, (unsigned long long)a.cap);
+    const uint32_t above = (uint32_t)max((unsigned long long)kCoopMin, K / kCoopLists + 1ull);
+    const long long cand = min((long long)coff[claim_class(above) + 1], a.G);
+    if (cand > 0) {
+        coop_collect<kTlThreads>(a, s_coop, coff, cand, above, K);
+        if (s_coop.count > 0 && !coop_sort<kTlThreads>(a, s_coop, s, s_split)) return;
+    }
     for (long long i = blockIdx.x; i < nlong; i += a.long_blocks) {
         const long long g = claim_at(coff, a.clist, a.G, i);
         const uint2 rng = g < a.G ? reinterpret_cast<const uint2 *>(a.ranges)[g] : make_uint2(1u, 0u);
@@ -593,6 +810,7 @@ __global__ void __launch_bounds__(kTlThreads, 1024 / kTlThreads) k_tile_sort(Bin
         const long long s0 = rng.x;
         const int n = (int)(rng.y - rng.x);
         if (n <= kWarpSort) continue;     // exactly 256 words: a short list
+        if (rng.y - rng.x > above) continue;   // sorted above
         // (the words lie in the key buffer that is not the output)
         word_t *in = a.words + s0, *out = reinterpret_cast<word_t *>(kout) + s0;
         if (n <= kRun) {
@@ -610,58 +828,14 @@ __global__ void __launch_bounds__(kTlThreads, 1024 / kTlThreads) k_tile_sort(Bin
             for (int e = tid; e < len; e += kTlThreads) in[r0 + e] = s[pd(e)];
             __syncthreads();
         }
-        // merges of runs of w words, kRun outputs at a time
         const int nblk = (n + kRun - 1) / kRun;
         for (long long w = kRun; w < n; w <<= 1) {
-            auto group = [&](int b, int &base, int &na, int &nb) {
-                base = (int)((long long)b * kRun / (2 * w) * (2 * w));
-                na = (int)min(w, (long long)n - base);
-                nb = (int)min(w, (long long)n - base - na);
-            };
-            for (int b0 = 0; b0 < nblk; b0 += kTlThreads) {
-                for (int q = tid; q <= kTlThreads; q += kTlThreads) {   // where each block's outputs start in its first run
-                    const int b = b0 + q;
-                    if (b < nblk) {
-                        int base, na, nb;
-                        group(b, base, na, nb);
-                        s_split[q] = merge_split([&](int j) { return in[j]; }, base, na, base + na, nb, b * kRun - base);
-                    }
-                }
-                __syncthreads();
-                for (int b = b0; b < min(b0 + kTlThreads, nblk); ++b) {
-                    int base, na, nb;
-                    group(b, base, na, nb);
-                    const int d0 = b * kRun - base, d1 = min(d0 + kRun, na + nb);
-                    const int a0 = s_split[b - b0], a1 = d1 == na + nb ? na : s_split[b - b0 + 1];
-                    const int ca = a1 - a0, cb = d1 - d0 - ca, from = base + na + (d0 - a0);
-                    for (int e = tid; e < ca + cb; e += kTlThreads) s[pd(e)] = e < ca ? in[base + a0 + e] : in[from + e - ca];
-                    __syncthreads();
-                    word_t x[kTlKPT];
-                    const bool act = tid * kTlKPT < ca + cb;
-                    if (act) merge_regs<kTlKPT>(s, 0, ca, ca, cb, tid * kTlKPT, x);
-                    __syncthreads();
-                    if (act) {
-#pragma unroll
-                        for (int r = 0; r < kTlKPT; ++r) s[pd(tid * kTlKPT + r)] = x[r];
-                    }
-                    __syncthreads();
-                    for (int e = tid; e < ca + cb; e += kTlThreads) out[b * kRun + e] = s[pd(e)];
-                    __syncthreads();
-                }
-            }
+            for (int b = 0; b < nblk; ++b) merge_block<kTlThreads>(s, s_split, in, out, n, b, w);
             word_t *x = in;
             in = out;
             out = x;
         }
-        // kout may be either buffer: an entry's key is written by the thread that read its word, and the
-        // record copy takes the pair index from vout
-        for (int e = tid; e < n; e += kTlThreads) emit_entry(a, kout, vout, g, s0 + e, in[e]);
-        __syncthreads();
-        copy_records<kTlThreads>(a, s0, n, tid, [&](int e) {
-            const uint32_t f = vout[s0 + e], sl = (long long)f < a.P ? a.slot[f] : kNoSlot;
-            return sl < (unsigned long long)a.vcap ? sl : kNoSlot;
-        });
-        __syncthreads();
+        for (int r0 = 0; r0 < n; r0 += kRun) finish_run<kTlThreads>(a, s, in, g, s0, r0, min(kRun, n - r0));
     }
 }
 
@@ -696,8 +870,9 @@ static int launch_tile_sort(BinArgs a, cudaStream_t s) {
                                             (int)kTileSortSmem<THREADS>) == cudaSuccess;
     if (!attr) return GS_ERR_CUDA;
     constexpr int kWarps = THREADS / 32;
-    a.long_blocks = a.max_count > kWarpSort   // a view's Gaussians bound its lists
-                        ? std::min<long long>(a.G, (long long)device_sm_count() * (1024 / THREADS)) : 0;
+    // a view's Gaussians bound its lists; CTAs beyond the lists share them
+    a.long_blocks = a.max_count > kWarpSort ? (long long)device_sm_count() * (1024 / THREADS) : 0;
+    if (a.max_count <= kCoopMin) a.long_blocks = std::min(a.long_blocks, a.G);
     k_tile_sort<THREADS><<<(unsigned)(a.long_blocks + (a.G + kWarps - 1) / kWarps), THREADS, kTileSortSmem<THREADS>, s>>>(a);
     return GS_OK;
 }
@@ -740,7 +915,8 @@ static int run_tile_first(BinArgs a, cudaStream_t s) {
 // 198 / 268 / 287; 8 agents' rooms, 32 views (7.3M keys, 62 pairs per tile) 479 / 559 / 883; 4 views of a 1M
 // room (4.9M keys, 310 pairs per tile) 376 / 373 / 529; 8 views of it (10.9M keys) 846 / 733 / 1096; 4 views
 // of a 2M floor (8.0M keys, 620 pairs per tile) 1138 / 608 / 885.  So: up to 4M pairs, or as long as the lists
-// are short.  Pairs that could pile up in few tiles (a list is one CTA's work) always take the radix binning.
+// are short, on average: how the pairs fall into tiles is not known here, and a view may have them all in a few (the
+// sort then shares the long lists among its CTAs).  Beyond 16384 pairs per tile always the radix binning.
 constexpr long long kTileFirstPairs = 4000000, kShortListPairs = 128, kMaxPairsPerTile = 16384;
 
 int run_bin_sort(const BinArgs &a, cudaStream_t s) {

@@ -27,6 +27,7 @@ constexpr int kChunk = 256;            // (view, Gaussian) pairs per projection 
 constexpr int kEmitPart = 1024;        // pairs per partition of the depth-ordered emission
 constexpr int kMaxTilePasses = 4;
 constexpr uint32_t kEmitKeysMin = 512; // keys per work item of the tile-first emission, at the least
+constexpr int kCoopWords = 193;        // ticket and done words of the tile-first sort's shared lists
 constexpr unsigned long long kSpinLimit = 1ull << 21;  // bounded waits (x ~100 ns sleep)
 
 // counters inside the status block (zero between calls: every launch returns its own to zero)
@@ -83,7 +84,7 @@ struct Layout {
     long long scan_parts, sort_parts, chunks_total;
     int sort_mode, nb;                 // binning mode; records per staged render batch
     size_t o_status, o_views, o_proj, o_touched, o_scan_state, o_keys[2], o_vals[2], o_hist,
-        o_sort_state, o_ranges, o_tcnt, o_tscan, o_vscan, o_escan, o_extra, o_srec, o_g2d, o_pose_part, o_slot, o_clist, o_slane,
+        o_sort_state, o_ranges, o_tcnt, o_tscan, o_coop, o_vscan, o_escan, o_extra, o_srec, o_g2d, o_pose_part, o_slot, o_clist, o_slane,
         o_blk, total;
     size_t o_guard[kNumGuards];        // guard blocks after proj, touched, keys x2, vals x2, ranges,
                                        // the extra emission items, srec, g2d, the pose partials, the slots,
