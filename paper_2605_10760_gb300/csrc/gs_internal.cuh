@@ -27,7 +27,8 @@ constexpr int kChunk = 256;            // (view, Gaussian) pairs per projection 
 constexpr int kEmitPart = 1024;        // pairs per partition of the depth-ordered emission
 constexpr int kMaxTilePasses = 4;
 constexpr uint32_t kEmitKeysMin = 512; // keys per work item of the tile-first emission, at the least
-constexpr int kCoopWords = 193;        // ticket and done words of the tile-first sort's shared lists
+constexpr int kCoopHot = 193;          // ticket and done words of the tile-first sort's shared lists, then the emission's
+constexpr int kCoopWords = kCoopHot + 1;   //   note of a tile with many keys
 constexpr unsigned long long kSpinLimit = 1ull << 21;  // bounded waits (x ~100 ns sleep)
 
 // counters inside the status block (zero between calls: every launch returns its own to zero)

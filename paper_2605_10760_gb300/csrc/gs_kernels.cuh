@@ -93,7 +93,8 @@ struct BinArgs {
     uint2 *extra;                      // [extra_cap] further (chunk, portion) items of the emission
     uint32_t extra_cap, emit_keys;     // keys per emission item
     long long long_blocks;             // CTAs of the sort that take the long lists
-    uint32_t *coop;                    // [kCoopWords] ticket and done words of the lists that these CTAs sort together
+    uint32_t *coop;                    // [kCoopWords] ticket and done words of the lists that these CTAs sort together,
+                                       //   and the emission's note of a tile with many keys
     uint32_t *clist;                   // [kClaimClasses, G] out: the items of each claim class
 };
 
