@@ -25,6 +25,10 @@ namespace gs {
 constexpr unsigned long long kEmptyKey = ~0ull;
 constexpr int kKeyBits = 21;
 constexpr long long kKeyOff = 1LL << 20;
+// words of a set's 256-byte header beside the status (bytes 8 .. 15 are gs_voxset_status's)
+constexpr int kStoredOffset = 16;      // keys stored, as far as reported
+constexpr int kLongestOffset = 24;     // the largest number of pauses (VoxProbe) that a stored key has made
+constexpr uint32_t kPatience = 32;     // slots between two pauses of a key
 constexpr int kMaxRaySteps = 1 << 16;  // voxels after the first of one ray before it is flagged
 constexpr int kMaxBoxExtent = 64;      // voxels per axis of one Gaussian's box before it is flagged
 
@@ -78,45 +82,84 @@ struct VoxProbe {
         const unsigned long long m = (unsigned long long)h * 0xc2b2ae3du;
         mix = (uint32_t)m ^ (uint32_t)(m >> 32);
         block = home(s);
+        pos = first(s);
+    }
+    __device__ __forceinline__ uint32_t first(const VoxSet &s) const {
+        const uint32_t lo = (uint32_t)key, hi = (uint32_t)(key >> 32);
         const uint32_t place = ((hi >> 10) & 3u) | ((lo >> 19) & 4u) | ((lo << 3) & 8u);
-        pos = (place ^ mix) & s.pos;
+        return (place ^ mix) & s.pos;
     }
     __device__ __forceinline__ uint32_t home(const VoxSet &s) const { return __umulhi(mix * 0x27d4eb2fu, s.blocks + 1u); }
     __device__ __forceinline__ size_t slot(const VoxSet &s) const { return ((size_t)block << s.shift) | pos; }
-    // the next slot; false once all have been visited (`places` counts the places done)
-    __device__ __forceinline__ bool next(const VoxSet &s, uint32_t &places) {
+    // On to the next line; true at a pause: after every kPatience slots (the step is odd, so the low bits of the line's
+    // number come round) and where the lines have come round, at home.
+    __device__ __forceinline__ bool advance(const VoxSet &s) {
         block = (block + ((mix >> 5) | 1u)) & s.blocks;
-        if (block == home(s)) {
-            pos = (pos + 1u) & s.pos;
-            return ++places <= s.pos;
-        }
-        return true;
+        return ((block ^ home(s)) & (kPatience - 1u)) == 0u;
+    }
+    // At a pause: on to the next place if this is home; false once all have been visited.
+    __device__ __forceinline__ bool turn(const VoxSet &s) {
+        if (block != home(s)) return true;
+        pos = (pos + 1u) & s.pos;
+        return pos != first(s);
     }
 };
 
-__device__ __forceinline__ bool voxset_insert(const VoxSet &s, unsigned long long key) {
+template <class T>
+__device__ __forceinline__ volatile T *voxset_word(const VoxSet &s, int offset) {
+    return reinterpret_cast<volatile T *>(reinterpret_cast<char *>(s.status) + offset);
+}
+
+// Reports the keys that this CTA has stored since its last report (`taken`).
+__device__ __forceinline__ void voxset_report(const VoxSet &s, uint32_t *taken) {
+    const uint32_t n = atomicExch(taken, 0u);
+    if (n) atomicAdd((unsigned long long *)voxset_word<unsigned long long>(s, kStoredOffset), (unsigned long long)n);
+}
+
+// A key that pauses reports its CTA's keys and asks whether the set is full (every CTA reports the rest when it ends, so
+// that is known soon after the last slot was taken).  A full set changes no more: with an error recorded the key may
+// leave it, and otherwise only needs to know whether it is in there, for which it looks no further than any stored
+// key has come.  Without the two words it would walk the whole set, or a sixteenth of it after an error.  2^17 slots
+// offered 10 times as many keys 0.19 ms, 2^22 slots 4 times 2.1 ms, 2^25 slots 1.5 times 18 ms (0.05, 0.7 and 2.5 ms
+// into a set that holds them).  The count is kept by the CTA, not the thread: a lane that waits for a neighbour's key
+// could not report its own.  It costs the rays 4 % (8 views of 600 x 340, 488 -> 507 us timed alone).
+__device__ __forceinline__ void voxset_insert(const VoxSet &s, unsigned long long key, uint32_t *taken) {
     VoxProbe p(s, key);
-    uint32_t places = 0;
-    do {
+    uint32_t pauses = 0;
+    for (;;) {
         unsigned long long *slot = s.keys + p.slot(s);
         const unsigned long long cur = *slot;
-        if (cur == p.key) return true;
+        if (cur == p.key) return;
         if (cur == kEmptyKey) {
             const unsigned long long prev = atomicCAS(slot, kEmptyKey, p.key);
-            if (prev == kEmptyKey || prev == p.key) return true;
+            if (prev == kEmptyKey) {
+                if (pauses) {
+                    atomicMax((uint32_t *)voxset_word<uint32_t>(s, kLongestOffset), pauses);
+                    __threadfence();           // before the count that may fill the set
+                }
+                atomicAdd(taken, 1u);
+            }
+            if (prev == kEmptyKey || prev == p.key) return;
         }
-        // a set that was found full stays full: one place of every line is enough to give up again
-    } while (p.next(s, places) && (places == 0u || *(volatile int32_t *)s.status != GS_ERR_CAPACITY));
+        if (p.advance(s)) {
+            ++pauses;
+            voxset_report(s, taken);
+            if (*voxset_word<unsigned long long>(s, kStoredOffset) >= ((unsigned long long)s.blocks + 1ull) << s.shift) {
+                __threadfence();
+                if (*voxset_word<int32_t>(s, 0) != 0) return;
+                if (pauses > *voxset_word<uint32_t>(s, kLongestOffset)) break;
+            }
+            if (!p.turn(s)) break;
+        }
+    }
     atomicCAS(s.status, 0, GS_ERR_CAPACITY);
-    return false;
 }
 
 // `cur` is what the caller found in the first slot
 __device__ __forceinline__ bool voxset_contains(const VoxSet &s, VoxProbe p, unsigned long long cur) {
-    uint32_t places = 0;
     for (;;) {
         if (cur == p.key) return true;
-        if (cur == kEmptyKey || !p.next(s, places)) return false;
+        if (cur == kEmptyKey || (p.advance(s) && !p.turn(s))) return false;
         cur = s.keys[p.slot(s)];
     }
 }
@@ -130,7 +173,11 @@ __global__ void k_voxset_clear(unsigned long long *keys, long long capacity, int
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < capacity;
          i += (long long)gridDim.x * blockDim.x)
         keys[i] = kEmptyKey;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *status = 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        *status = 0;
+        *reinterpret_cast<unsigned long long *>(reinterpret_cast<char *>(status) + kStoredOffset) = 0ull;
+        *reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(status) + kLongestOffset) = 0u;
+    }
 }
 
 // One Gaussian per lane for the box, then the warp's voxels one per lane in turn, those of a box along z first:
@@ -139,6 +186,9 @@ __global__ void k_voxset_clear(unsigned long long *keys, long long capacity, int
 // a box per lane and voxels hashed one by one.
 __global__ void __launch_bounds__(256) k_add_boxes(VoxSet s, long long n, const float *means, const float *log_scales,
                                                    float k, float v) {
+    __shared__ uint32_t s_taken;
+    if (threadIdx.x == 0) s_taken = 0u;
+    __syncthreads();
     const int lane = threadIdx.x & 31;
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long i0 = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); i0 < n; i0 += stride) {
@@ -182,10 +232,12 @@ __global__ void __launch_bounds__(256) k_add_boxes(VoxSet s, long long n, const 
                 const int ny = d >> 8, nz = d & 255;
                 const int row = (int)__fdividef((float)at + 0.5f, (float)nz), z = at - row * nz;
                 const int x = (int)__fdividef((float)row + 0.5f, (float)ny), y = row - x * ny;
-                voxset_insert(s, vox_key(x0 + x, y0 + y, z0 + z));
+                voxset_insert(s, vox_key(x0 + x, y0 + y, z0 + z), &s_taken);
             }
         }
     }
+    __syncthreads();
+    if (threadIdx.x == 0) voxset_report(s, &s_taken);
 }
 
 struct RayArgs {
@@ -204,6 +256,9 @@ struct RayArgs {
 // only after the next one's load was issued: 650 us (more instructions, and more slots found empty that another
 // warp had just filled).
 __global__ void __launch_bounds__(256, 8) k_add_rays(RayArgs a) {
+    __shared__ uint32_t s_taken;
+    if (threadIdx.x == 0) s_taken = 0u;
+    __syncthreads();
     const long long total = (long long)a.V * a.pw * a.ph * 32;
     for (long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x; r < total; r += (long long)gridDim.x * blockDim.x) {
         const int lane = threadIdx.x & 31;
@@ -247,7 +302,7 @@ __global__ void __launch_bounds__(256, 8) k_add_rays(RayArgs a) {
             }
         }
         unsigned long long key = vox_key(cur[0], cur[1], cur[2]);
-        voxset_insert(a.s, key);
+        voxset_insert(a.s, key, &s_taken);
         int n = 0;
         // A ray that starts far enough inside the range of keys never meets its limits: its key moves by the
         // step's own bits.
@@ -266,7 +321,7 @@ __global__ void __launch_bounds__(256, 8) k_add_rays(RayArgs a) {
                 tmax[0] = !q2 && !b1 ? n0 : tmax[0];
                 tmax[1] = !q2 && b1 ? n1 : tmax[1];
                 tmax[2] = q2 ? n2 : tmax[2];
-                voxset_insert(a.s, key);
+                voxset_insert(a.s, key, &s_taken);
             }
         } else {
             for (; n < kMaxRaySteps; ++n) {
@@ -280,11 +335,13 @@ __global__ void __launch_bounds__(256, 8) k_add_rays(RayArgs a) {
                         cur[d] += step[d];
                         tmax[d] = fp::add(tmax[d], tdel[d]);
                     }
-                voxset_insert(a.s, vox_key(cur[0], cur[1], cur[2]));
+                voxset_insert(a.s, vox_key(cur[0], cur[1], cur[2]), &s_taken);
             }
         }
         if (n == kMaxRaySteps) atomicCAS(a.s.status, 0, GS_ERR_INVALID_ARG);   // ray longer than allowed
     }
+    __syncthreads();
+    if (threadIdx.x == 0) voxset_report(a.s, &s_taken);
 }
 
 __global__ void k_keep(long long n, const float *means, VoxSet occ, VoxSet fre, bool has_free, float v,
