@@ -155,11 +155,15 @@ __device__ __forceinline__ void voxset_insert(const VoxSet &s, unsigned long lon
     atomicCAS(s.status, 0, GS_ERR_CAPACITY);
 }
 
-// `cur` is what the caller found in the first slot
+// `cur` is what the caller found in the first slot.  Up to the first empty slot, or as far as any stored key has come:
+// an overfull set has no empty slot, and a key that is not in it would be compared with all the others.  (1 M Gaussians
+// outside a set of 2^22 slots: 0.04 ms half full, 0.13 ms at 94 %, 2.6 ms overfull.)
 __device__ __forceinline__ bool voxset_contains(const VoxSet &s, VoxProbe p, unsigned long long cur) {
+    uint32_t pauses = 0;
     for (;;) {
         if (cur == p.key) return true;
-        if (cur == kEmptyKey || (p.advance(s) && !p.turn(s))) return false;
+        if (cur == kEmptyKey) return false;
+        if (p.advance(s) && (++pauses > *voxset_word<uint32_t>(s, kLongestOffset) || !p.turn(s))) return false;
         cur = s.keys[p.slot(s)];
     }
 }

@@ -71,3 +71,16 @@ def test_a_set_filled_to_the_last_slot_is_no_error(cap):
     s.clear()
     s.add_boxes(means[:cap], small[:cap], 3.0, V)
     assert s.status() == (0, cap)
+
+
+def test_asking_an_overfull_set_does_not_walk_it():
+    """(A million absent keys against all four million stored ones would take minutes.)"""
+    from paper_2605_10760_gb300 import _lib as L, raster as R
+    cap, offered = 1 << 22, 9 << 19
+    means = centres(offered + (1 << 20), 5)
+    s = R.VoxSet(cap)
+    s.add_boxes(means[:offered], torch.full((offered, 3), -12.0, device="cuda"), 3.0, V)
+    assert s.status() == (L.GS_ERR_CAPACITY, cap)
+    keep = torch.empty(len(means), dtype=torch.uint8, device="cuda")
+    assert timed(lambda: keep.copy_(R.dedup_keep(means, s, None, V))) < 0.3
+    assert int((keep == 0).sum()) == cap and bool(keep[offered:].all())
