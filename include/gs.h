@@ -516,6 +516,10 @@ int64_t gs_launch_count(void);
  * (either output may be NULL).  n elements, device arrays. */
 int gs_debug_expf(const float *x, float *y_spec, float *y_cuda, int64_t n, void *stream);
 
+/* The same exponential in the packed forms that the compositing kernels evaluate for two pixels at
+ * once: y_packed for any argument, y_neg for arguments in [-80, 0] (others give garbage there). */
+int gs_debug_exp2(const float *x, float *y_packed, float *y_neg, int64_t n, void *stream);
+
 /* Bounded-wait check of the decoupled look-back: runs the inclusive scan over n ones in `scratch`
  * (device, gs_debug_scan_scratch_size(n) bytes) with partition `silent_partition` never
  * publishing its count (-1: normal run) and a short spin limit (about a millisecond), then

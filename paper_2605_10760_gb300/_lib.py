@@ -172,6 +172,7 @@ _SIGS = {
     "gs_grads_zero": (C.c_int, [C.c_int64, C.POINTER(gs_grads), _P]),
     "gs_launch_count": (C.c_int64, []),
     "gs_debug_expf": (C.c_int, [_P, _P, _P, C.c_int64, _P]),
+    "gs_debug_exp2": (C.c_int, [_P, _P, _P, C.c_int64, _P]),
     "gs_debug_scan_scratch_size": (C.c_size_t, [C.c_int64]),
     "gs_debug_scan_timeout": (C.c_int, [_P, C.c_int64, C.c_int32, _P, C.POINTER(C.c_int64)]),
 }

@@ -830,6 +830,20 @@ __global__ void k_debug_expf(const float *x, float *ys, float *yc, long long n) 
     }
 }
 
+// element i as one half of a pair with element i ^ 1
+__global__ void k_debug_exp2(const float *x, float *yp, float *yn, long long n) {
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; 2 * i < n; i += (long long)gridDim.x * blockDim.x) {
+        const float2 v = make_float2(x[2 * i], 2 * i + 1 < n ? x[2 * i + 1] : 0.f);
+        const float2 p = spec_expf2(v), q = spec_exp_neg(fp2::neg(v));
+        yp[2 * i] = p.x;
+        yn[2 * i] = q.x;
+        if (2 * i + 1 < n) {
+            yp[2 * i + 1] = p.y;
+            yn[2 * i + 1] = q.y;
+        }
+    }
+}
+
 int gs_grads_zero(int64_t n, const gs_grads *g, void *stream) {
     GS_RANGE("gs_grads_zero");
     if (n < 0 || !g) return GS_ERR_INVALID_ARG;
@@ -845,6 +859,15 @@ int gs_debug_expf(const float *x, float *y_spec, float *y_cuda, int64_t n, void 
     if (n == 0) return GS_OK;
     const int grid = (int)std::min<long long>((n + 255) / 256, 4096);
     k_debug_expf<<<grid, 256, 0, (cudaStream_t)stream>>>(x, y_spec, y_cuda, n);
+    count_launches(1);
+    return check_launch();
+}
+
+int gs_debug_exp2(const float *x, float *y_packed, float *y_neg, int64_t n, void *stream) {
+    if (!x || !y_packed || !y_neg || n < 0) return GS_ERR_INVALID_ARG;
+    if (n == 0) return GS_OK;
+    const int grid = (int)std::min<long long>((n + 511) / 512, 4096);
+    k_debug_exp2<<<grid, 256, 0, (cudaStream_t)stream>>>(x, y_packed, y_neg, n);
     count_launches(1);
     return check_launch();
 }

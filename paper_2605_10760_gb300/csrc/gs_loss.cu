@@ -142,7 +142,7 @@ static SsimTaps make_taps() {
 // the two components of packed FP32x2 arithmetic: pass 1 filters (x, y) and (x^2, y^2) packed and x y alone, pass
 // 2 (dS/dmu_x, dS/dE[x^2]) packed and dS/dE[xy] alone.  (The SSIM map's mean enters an FP64 loss and its bias
 // comes from the rounding of these sums, so their operations are part of the result: taps in ascending order,
-// w x rounded before it is added or meets its second factor.)  The pitches below and the order of the lanes in
+// w x rounded before it is added or meets its second factor; used twice, it is not joined with the sum.)  The pitches below and the order of the lanes in
 // the horizontal filter (hlane) keep every 16-byte shared access of eight lanes on 32 different banks.
 // 8 views of 1200 x 680 (19.6 M samples): pass 1 187 us (68 % of the issue slots; 392 MB take 58 us), pass 2 142 us
 // (62 %; 470 MB, 69 us); tiles of 32 x 32 on their own 213 and 173 us; with one sample per load and scalar
