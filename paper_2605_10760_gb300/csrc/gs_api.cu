@@ -26,16 +26,18 @@ int check_launch() {
     return e == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }
 
+int current_device() {
+    int dev = -1;
+    return cudaGetDevice(&dev) == cudaSuccess ? dev : -1;
+}
+
 int device_sm_count() {
-    static int cache[64] = {0};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 1;
-    if (!cache[dev]) {
+    static PerDevice count;
+    const int dev = current_device();
+    return std::max(1, count.get(dev, [&] {
         int n = 0;
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        cache[dev] = n > 0 ? n : 1;
-    }
-    return cache[dev];
+        return dev >= 0 && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess ? n : 0;
+    }));
 }
 
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }

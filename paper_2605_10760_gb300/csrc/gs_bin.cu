@@ -914,8 +914,11 @@ static int occupancy(const void *fn, int threads) {
 // (a.chunks > 0)
 void launch_scan_chunks(const BinArgs &a, bool pairs, cudaStream_t s) {
     const long long parts = (a.chunks + kScanTile - 1) / kScanTile;
-    static int occ = std::min(occupancy((const void *)k_scan_chunks<true>, kCsThreads),
-                              occupancy((const void *)k_scan_chunks<false>, kCsThreads));
+    static PerDevice per;
+    const int occ = per.get(current_device(), [] {
+        return std::min(occupancy((const void *)k_scan_chunks<true>, kCsThreads),
+                        occupancy((const void *)k_scan_chunks<false>, kCsThreads));
+    });
     const unsigned grid = (unsigned)std::min<long long>(parts, (long long)device_sm_count() * occ);
     if (pairs) k_scan_chunks<true><<<grid, kCsThreads, 0, s>>>(a);
     else k_scan_chunks<false><<<grid, kCsThreads, 0, s>>>(a);
@@ -929,9 +932,12 @@ void launch_claims(const BinArgs &a, cudaStream_t s) {
 
 template <int THREADS>
 static int launch_tile_sort(BinArgs a, cudaStream_t s) {
-    static bool attr = cudaFuncSetAttribute((const void *)k_tile_sort<THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)kTileSortSmem<THREADS>) == cudaSuccess;
-    if (!attr) return GS_ERR_CUDA;
+    static PerDevice attr;
+    if (!attr.get(current_device(), [] {
+            return cudaFuncSetAttribute((const void *)k_tile_sort<THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)kTileSortSmem<THREADS>) == cudaSuccess;
+        }))
+        return GS_ERR_CUDA;
     constexpr int kWarps = THREADS / 32;
     // a view's Gaussians bound its lists; CTAs beyond the lists share them
     a.long_blocks = a.max_count > kWarpSort ? (long long)device_sm_count() * (1024 / THREADS) : 0;
@@ -957,10 +963,12 @@ static int run_tile_first(BinArgs a, cudaStream_t s) {
     }
     BinArgs t = a;
     t.scan_state = a.tile_scan_state;
-    static int occ_t = occupancy((const void *)k_tile_scan, kCsThreads);
+    static PerDevice per_t, per_s;
+    const int dev = current_device();
+    const int occ_t = per_t.get(dev, [] { return occupancy((const void *)k_tile_scan, kCsThreads); });
     const long long gparts = (a.G + kScanTile - 1) / kScanTile;
     k_tile_scan<<<(unsigned)std::min<long long>(gparts, sms * occ_t), kCsThreads, 0, s>>>(t);
-    static int occ_s = occupancy((const void *)k_scatter, kScThreads);
+    const int occ_s = per_s.get(dev, [] { return occupancy((const void *)k_scatter, kScThreads); });
     k_scatter<<<(unsigned)std::max<long long>(1, std::min<long long>((a.cap + kScThreads - 1) / kScThreads, sms * occ_s)),
                 kScThreads, 0, s>>>(a);
     // fewer tiles than SMs: a CTA of 1024 threads per list, whose runs hold 8192 words, else 256 threads

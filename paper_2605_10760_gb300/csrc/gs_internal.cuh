@@ -11,6 +11,7 @@
 #include <stdint.h>
 
 #include "../../include/gs.h"
+#include "gs_device.cuh"
 
 namespace gs {
 
@@ -471,6 +472,7 @@ int compute_layout(const gs_problem *pb, Layout *L);
 // scans the guard blocks (synchronises the stream); *first_bad = index of the first changed block or -1
 int run_check_guards(const unsigned char *const *guards, DevStatus *st, int32_t *first_bad, cudaStream_t s);
 void count_launches(int n);
+int current_device();        // -1 without one
 int device_sm_count();
 int check_launch();
 

@@ -794,7 +794,8 @@ static int persistent_grid(F fn, int threads) {
 template <int TW, int TH, int NB>
 static int fwd_t(const FwdArgs &a, cudaStream_t s) {
     constexpr int NT = TW * TH / kPPT;
-    static int grid = persistent_grid(k_render_fwd<TW, TH, NB>, NT);
+    static PerDevice per;
+    const int grid = per.get(current_device(), [] { return persistent_grid(k_render_fwd<TW, TH, NB>, NT); });
     if (a.rgb_t && cudaMemsetAsync(a.loss, 0, sizeof(double), s) != cudaSuccess) return GS_ERR_CUDA;
     const long long g = std::min<long long>(grid, std::max<long long>(1, a.G));
     k_render_fwd<TW, TH, NB><<<(unsigned)g, NT, 0, s>>>(a);
@@ -805,7 +806,8 @@ static int fwd_t(const FwdArgs &a, cudaStream_t s) {
 template <int TW, int TH, int NB>
 static int bwd_t(const BwdArgs &a, cudaStream_t s) {
     constexpr int NT = TW * TH / kPPT;
-    static int grid = persistent_grid(k_render_bwd<TW, TH, NB>, NT);
+    static PerDevice per;
+    const int grid = per.get(current_device(), [] { return persistent_grid(k_render_bwd<TW, TH, NB>, NT); });
     const long long g = std::min<long long>(grid, std::max<long long>(1, a.G));
     k_render_bwd<TW, TH, NB><<<(unsigned)g, NT, 0, s>>>(a);
     count_launches(1);

@@ -535,7 +535,8 @@ int run_scan_only(const BinArgs &a, cudaStream_t s) {
     const long long parts = (a.P + kScanTile - 1) / kScanTile;
     if (parts > 0) {
         if (cudaMemsetAsync(a.scan_state, 0, sizeof(unsigned long long) * parts, s) != cudaSuccess) return GS_ERR_CUDA;
-        static int occ = occupancy((const void *)k_scan, kScanThreads, 0);
+        static PerDevice per;
+        const int occ = per.get(current_device(), [] { return occupancy((const void *)k_scan, kScanThreads, 0); });
         long long grid = std::min<long long>(parts, (long long)device_sm_count() * occ);
         k_scan<<<(unsigned)grid, kScanThreads, 0, s>>>(a);
         count_launches(1);
@@ -547,10 +548,14 @@ int run_scan_only(const BinArgs &a, cudaStream_t s) {
 }
 
 static int sweep(const BinArgs &a, SweepArgs sa, int pass, cudaStream_t s) {
-    static bool attr = cudaFuncSetAttribute((const void *)k_onesweep<kSortIPT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)sweep_dyn_smem<kSortIPT>()) == cudaSuccess;
-    if (!attr) return GS_ERR_CUDA;
-    static int occ = occupancy((const void *)k_onesweep<kSortIPT>, kSortThreads, sweep_dyn_smem<kSortIPT>());
+    static PerDevice attr, per;
+    const int dev = current_device();
+    if (!attr.get(dev, [] {
+            return cudaFuncSetAttribute((const void *)k_onesweep<kSortIPT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)sweep_dyn_smem<kSortIPT>()) == cudaSuccess;
+        }))
+        return GS_ERR_CUDA;
+    const int occ = per.get(dev, [] { return occupancy((const void *)k_onesweep<kSortIPT>, kSortThreads, sweep_dyn_smem<kSortIPT>()); });
     const long long grid = std::max<long long>(1, std::min<long long>(a.sort_parts, (long long)device_sm_count() * occ));
     sa.hist = a.hist + 256 * pass;
     sa.state = a.sort_state + (size_t)256 * a.sort_parts * pass;
@@ -569,7 +574,9 @@ int run_onesweep(const BinArgs &a, cudaStream_t s) {
     if (cudaMemsetAsync(a.clear_begin, 0, a.clear_bytes, s) != cudaSuccess) return GS_ERR_CUDA;
     const long long sms = device_sm_count();
     launch_scan_chunks(a, true, s);
-    static int occ_c = occupancy((const void *)k_compact, kCpThreads, 0);
+    static PerDevice per_c, per_e;
+    const int dev = current_device();
+    const int occ_c = per_c.get(dev, [] { return occupancy((const void *)k_compact, kCpThreads, 0); });
     k_compact<<<(unsigned)std::max<long long>(1, std::min<long long>((a.chunks + 7) / 8, sms * occ_c)), kCpThreads, 0, s>>>(a);
     count_launches(1);
     SweepArgs sa;
@@ -586,7 +593,7 @@ int run_onesweep(const BinArgs &a, cudaStream_t s) {
     }
     BinArgs e = a;
     e.scan_state = a.emit_scan_state;
-    static int occ_e = occupancy((const void *)k_emit_sorted, kEsThreads, 0);
+    const int occ_e = per_e.get(dev, [] { return occupancy((const void *)k_emit_sorted, kEsThreads, 0); });
     const long long parts = std::max<long long>(1, (std::min(a.cap, a.P) + kEmitPart - 1) / kEmitPart);
     k_emit_sorted<<<(unsigned)std::min<long long>(parts, sms * occ_e), kEsThreads, 0, s>>>(e);
     count_launches(1);
