@@ -281,10 +281,10 @@ __device__ __forceinline__ float spec_sigma(float A, float B, float C, float dx,
 // round each component exactly like the scalar operation, so every component equals the scalar
 // chain's result bit for bit.  One thing has to be watched: the assembler joins a packed product
 // and a packed sum that is its only use into one fused operation, although both state their
-// rounding (it does not join scalar products, nor a product that is used again).  The one such pair
-// of the chain, in the exponential, takes two scalar products (mul1): joined, 9 floats of [0, 80]
-// came out one unit in the last place off, and compositing 32 views took 0.4 % less (1102 for 1107
-// us forward, 2089 for 2099 backward; a product a b - 0 with the zero read at run time 1126, 2107).
+// rounding (it does not join a product that is used again).  The one such pair of the chain, in the
+// exponential, takes the product as a b + 0 (mul0): joined, 9 floats of [0, 80] came out one unit in
+// the last place off.  (Compositing 32 views, forward and backward: 1102 and 2089 us joined, 1101 and
+// 2092 with a b + 0, 1107 and 2098 with two scalar products, 1126 and 2107 with a zero read at run time.)
 // ------------------------------------------------------------------------------------------
 namespace fp2 {
 __device__ __forceinline__ float2 splat(float a) { return make_float2(a, a); }
@@ -292,7 +292,8 @@ __device__ __forceinline__ float2 neg(float2 a) { return make_float2(-a.x, -a.y)
 __device__ __forceinline__ float2 mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 add(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 mul1(float2 a, float b) { return make_float2(fp::mul(a.x, b), fp::mul(a.y, b)); }
+// a b for a sum with anything but a zero (a product of -0 comes out as +0)
+__device__ __forceinline__ float2 mul0(float2 a, float b) { return fma(a, splat(b), splat(0.f)); }
 }  // namespace fp2
 
 // spec_expf of both components (a - b is computed as a + (-b) and (-k) c as k (-c), both exact)
@@ -301,7 +302,7 @@ __device__ __forceinline__ float2 spec_expf2(float2 x) {
     const float kLn2Hi = 0x1.62e4p-1f;
     const float kLn2Lo = 0x1.7f7d1cp-20f;
     const float kShift = 12582912.0f;
-    const float2 t = fp2::add(fp2::mul1(x, kLog2e), fp2::splat(kShift));
+    const float2 t = fp2::add(fp2::mul0(x, kLog2e), fp2::splat(kShift));
     const float2 kf = fp2::add(t, fp2::splat(-kShift));
     float2 r = fp2::fma(kf, fp2::splat(-kLn2Hi), x);
     r = fp2::fma(kf, fp2::splat(-kLn2Lo), r);
@@ -336,7 +337,7 @@ __device__ __forceinline__ double pair_value(float2 s) { return isinf(s.x) ? (do
 __device__ __forceinline__ float2 spec_exp_neg(float2 s) {
     using fp2::splat;
     const float kShift = 12582912.0f;
-    const float2 t = fp2::add(fp2::mul1(s, -0x1.715476p+0f), splat(kShift));
+    const float2 t = fp2::add(fp2::mul0(s, -0x1.715476p+0f), splat(kShift));
     const float2 kf = fp2::add(t, splat(-kShift));
     float2 r = fp2::fma(kf, splat(0x1.62e4p-1f), s);         // -r of spec_expf
     r = fp2::fma(kf, splat(0x1.7f7d1cp-20f), r);

@@ -51,8 +51,7 @@ __device__ void pho_quat_matrix(const float *qin, float *M) {
 }
 
 // The rounded product a b as a b - 0 (nz: -0 in both halves, read at run time): the assembler joins a packed
-// product and a packed sum that is its only use into one fused operation, which the chain must not have.  (Two
-// scalar products, as the compositing takes for its one such pair, would be an instruction more for each of these.)
+// product and a packed sum that is its only use into one fused operation, which the chain must not have.
 __device__ __forceinline__ float2 mul2(float2 a, float2 b, float2 nz) { return fp2::fma(a, b, nz); }
 
 // (M v)_i = (M_i0 v_0 + M_i1 v_1) + M_i2 v_2 and the transposed form, every operation rounded.
