@@ -72,7 +72,8 @@ typedef struct gs_camera {
  *   Tile-first: the keys of every tile are counted, a scan of the G counts gives each tile its slice,
  *     every key is dropped into its slice as the word (depth bits, pair index) in arbitrary order and
  *     each slice is sorted on chip (a warp per slice of at most 256 words, a CTA per longer one, slices
- *     longer than 4096 words as sorted runs merged in global memory).  Faster for few or short lists.
+ *     longer than 2048 words, or 8192 where the tiles are no more than the SMs, as sorted runs merged in
+ *     global memory, the longest slices by all CTAs together).  Faster for few or short lists.
  *   Radix: the visible pairs sorted by depth, their keys emitted in that order and sorted by tile, both
  *     by a stable LSD onesweep radix sort (at most 8-bit digits, decoupled look-back).  Faster for many
  *     long lists.

@@ -30,8 +30,9 @@ constexpr int kCsThreads = 1024, kCsIPT = 4;
 static_assert(kCsThreads * kCsIPT == kScanTile, "the layout sizes the look-back words by kScanTile");
 
 // blk[c].z = keys of chunk c -> blk[c].w = keys of the chunks before it (saturated at 2^32 - 1, far
-// above any capacity).  PAIRS: blk[c].z then becomes the visible pairs before it.  Otherwise a chunk with more than a.emit_keys keys also lists its further portions of
-// that many keys as extra work items of k_emit_tiles (those that start below the capacity).
+// above any capacity).  PAIRS: blk[c].z then becomes the visible pairs before it.  Otherwise a chunk with more than
+// a.emit_keys keys also lists its further portions of that many keys as extra work items of k_emit_tiles (those that
+// start below the capacity).
 template <bool PAIRS>
 __global__ void __launch_bounds__(kCsThreads) k_scan_chunks(BinArgs a) {
     __shared__ uint32_t s_part;
@@ -56,12 +57,12 @@ __global__ void __launch_bounds__(kCsThreads) k_scan_chunks(BinArgs a) {
             tsum += x[k];
             vsum += nv[k];
         }
-        unsigned long long run = scan_partition<kCsThreads>(a, sh, part, nparts, tsum, [] {});
+        unsigned long long run = scan_partition<kCsThreads>(a, sh, part, nparts, tsum);
         if constexpr (PAIRS) {
             __syncthreads();              // sh.prefix has been read
             BinArgs av = a;
             av.scan_state = a.vis_scan_state;
-            unsigned long long vrun = scan_partition<kCsThreads, false>(av, sh, part, nparts, vsum, [] {});
+            unsigned long long vrun = scan_partition<kCsThreads, false>(av, sh, part, nparts, vsum);
             if (part == nparts - 1 && threadIdx.x == kCsThreads - 1) a.st->bin_pairs = vrun + vsum;
 #pragma unroll
             for (int k = 0; k < kCsIPT; ++k) {
@@ -304,7 +305,7 @@ __global__ void __launch_bounds__(kCsThreads) k_tile_scan(BinArgs a) {
             tsum += x[k];
             pos[k] = class_position(s_cls, claim_class(x[k]), base + k < a.G);
         }
-        unsigned long long run = scan_partition<kCsThreads, false>(a, sh, part, nparts, tsum, [] {});
+        unsigned long long run = scan_partition<kCsThreads, false>(a, sh, part, nparts, tsum);
         if (threadIdx.x < kClaimClasses) {
             const uint32_t c = s_cls[threadIdx.x];
             s_base[threadIdx.x] = c ? atomicAdd(&a.st->claim_cnt[threadIdx.x], c) : 0u;

@@ -77,7 +77,8 @@ struct VoxProbe {
     __device__ __forceinline__ VoxProbe(const VoxSet &s, unsigned long long k) : key(k) {
         const uint32_t lo = (uint32_t)k, hi = (uint32_t)(k >> 32);   // y's low 11 bits and z; x and y's high 10 bits
         // the block (two bits of x, one of y and z masked off) through odd multipliers, then a multiplication
-        // whose halves are folded onto each other, and the high part of another one
+        // whose halves are folded onto each other, and the high part of another one (the multipliers are primes
+        // of xxHash32)
         const uint32_t h = (lo & ~0x00200001u) * 0x9e3779b1u + (hi & ~0x00000c00u) * 0x85ebca77u;
         const unsigned long long m = (unsigned long long)h * 0xc2b2ae3du;
         mix = (uint32_t)m ^ (uint32_t)(m >> 32);

@@ -100,8 +100,8 @@ struct BinArgs {
 
 // Either way the sorted keys end in keys[passes % 2], the values in vals[passes % 2], the records in
 // list order in srec.  run_bin_sort chooses: tile-first (gs_bin.cu: keys into tile slices, every slice
-// sorted on chip) or run_onesweep (gs_sort.cu: scan with key emission and digit histograms -> onesweep
-// passes -> ranges).
+// sorted on chip) or run_onesweep (gs_sort.cu: the visible pairs sorted by depth, their keys emitted in
+// that order and sorted by tile, then ranges and records).
 int run_bin_sort(const BinArgs &a, cudaStream_t s);
 int run_onesweep(const BinArgs &a, cudaStream_t s);
 void launch_scan_chunks(const BinArgs &a, bool pairs, cudaStream_t s);

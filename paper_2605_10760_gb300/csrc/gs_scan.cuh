@@ -21,12 +21,10 @@ struct ScanShared {
 // the thread's counts (threads in order).  Block scan of the per-thread sums; warp 0 publishes the
 // partition total, looks back over the predecessors (a warp reads 32 at a time, the nearest
 // inclusive word ends it; bounded spins) and publishes the inclusive prefix; the last partition
-// writes K and checks the capacity (TOTAL).  Every thread runs `overlap` (work that needs no prefix) before
-// the closing barrier, warp 0 after its look-back.  sh.prefix holds the partition's prefix on
-// return.
-template <int THREADS, bool TOTAL = true, class Overlap>
+// writes K and checks the capacity (TOTAL).  sh.prefix holds the partition's prefix on return.
+template <int THREADS, bool TOTAL = true>
 __device__ unsigned long long scan_partition(const BinArgs &a, ScanShared<THREADS> &sh, long long part,
-                                             long long nparts, unsigned long long tsum, Overlap &&overlap) {
+                                             long long nparts, unsigned long long tsum) {
     static_assert(THREADS / 32 <= 32, "warp 0 scans the warp sums");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     unsigned long long incl = tsum;
@@ -94,7 +92,6 @@ __device__ unsigned long long scan_partition(const BinArgs &a, ScanShared<THREAD
             }
         }
     }
-    overlap();   // work that needs no prefix: warps 1.. while warp 0 looks back, warp 0 after it
     __syncthreads();
     return sh.prefix + sh.wsum[warp] + (incl - tsum);
 }

@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(BinArgs a) {
         unsigned long long tsum = 0;
 #pragma unroll
         for (int k = 0; k < kScanIPT; ++k) tsum += x[k];
-        unsigned long long run = scan_partition<kScanThreads>(a, sh, part, nparts, tsum, [] {});
+        unsigned long long run = scan_partition<kScanThreads>(a, sh, part, nparts, tsum);
         uint32_t y[kScanIPT];
 #pragma unroll
         for (int k = 0; k < kScanIPT; ++k) {
@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(kEsThreads) k_emit_sorted(BinArgs a) {
             x[k] = s_inc[tid * kEsIPT + k];
             tsum += x[k];
         }
-        unsigned long long run = scan_partition<kEsThreads, false>(a, sh, part, nparts, tsum, [] {});
+        unsigned long long run = scan_partition<kEsThreads, false>(a, sh, part, nparts, tsum);
         const unsigned long long pstart = sh.prefix;
 #pragma unroll
         for (int k = 0; k < kEsIPT; ++k) {
