@@ -270,8 +270,9 @@ constexpr int kResident = (kWide<TW, TH, NB> ? 2048 : 2560) / (TW * TH);
 // they are only while the entry's colour and depth and the pixel's upstream gradient are tame: 0 x NaN is NaN, and a
 // lane whose quarter has no entry left reads another entry of the batch.  The projection gives other entries an
 // infinite cut-off, and their batches (and, in the backward, those of a tile with other gradients) take the SLOW
-// walk, in which a pixel's sums meet only the entries that it blends.  The gradients are looked at once a batch: a
-// flag kept through the walk cost the backward of short lists 1 % (32 views, 7.3M list entries: 2119 for 2093 us).
+// walk, in which a pixel's sums meet only the entries that it blends.  The backward of short lists looks at the
+// gradients once a batch: a flag kept through the walk cost it 1 % (32 views, 7.3M list entries: 2119 for 2093 us).
+// That of long lists keeps the flag: a look per batch cost it 2 % (8 views, 10.7M: 2247 for 2201 us).
 __device__ __forceinline__ float2 select2(bool x, bool y, float2 a, float2 b) {
     return make_float2(x ? a.x : b.x, y ? a.y : b.y);
 }
@@ -622,6 +623,10 @@ __global__ void __launch_bounds__(TW *TH / kPPT, kResident<TW, TH, NB>) k_render
         const float2 py = make_float2((float)y0 + 0.5f, (float)(y0 + 1) + 0.5f);
         const int wmax = __reduce_max_sync(0xffffffffu, tmax);
         if (lane == 0) atomicMax(&sm.maxlast, wmax);
+        bool bent = false;                 // (kWide) the warp's gradients or sums are not tame
+        if constexpr (kWide<TW, TH, NB>)
+            bent = __any_sync(0xffffffffu, !(tame(tC0[0], tC1[0], tC2[0], tD[0]) && tame(tC0[1], tC1[1], tC2[1], tD[1]) &&
+                                             tame(tQ[0], tQ[1], 0.f, 0.f)));
         // the quarter's largest last index
         int qmax = tmax;
 #pragma unroll
@@ -768,12 +773,18 @@ __global__ void __launch_bounds__(TW *TH / kPPT, kResident<TW, TH, NB>) k_render
             }
             parity[buf] ^= 1u;
             const float4 *rec = sm.rec[buf];
-            const bool calm = tame(gC0.x, gC1.x, gC2.x, gD.x) && tame(gC0.y, gC1.y, gC2.y, gD.y) && tame(Q.x, Q.y, 0.f, 0.f);
+            bool calm = true;
+            if constexpr (!kWide<TW, TH, NB>)
+                calm = tame(gC0.x, gC1.x, gC2.x, gD.x) && tame(gC0.y, gC1.y, gC2.y, gD.y) && tame(Q.x, Q.y, 0.f, 0.f);
             const bool slow = __syncthreads_or(stage_masks<TW, TH, NB>(rec, sm.mask, cnt, tx * TW, ty * TH) | !calm);
             // entries at or beyond the warp's largest last_idx contribute nothing to this warp
             const int kend = min(hi, wmax) - lo;
-            if (slow) walk(std::true_type(), rec, sm.mask, lo, kend);
-            else walk(std::false_type(), rec, sm.mask, lo, kend);
+            if (slow || bent) {
+                walk(std::true_type(), rec, sm.mask, lo, kend);
+                if constexpr (kWide<TW, TH, NB>) bent = bent || __any_sync(0xffffffffu, !tame(Q.x, Q.y, 0.f, 0.f));
+            } else {
+                walk(std::false_type(), rec, sm.mask, lo, kend);
+            }
             __syncthreads();                          // buffer reads finished before its refill
             buf ^= 1;
         }

@@ -148,3 +148,31 @@ def test_gradients_beside_a_colour_and_an_upstream_value(R, shape, bad):
         bent[a][pick] = bad
         pb, g, img = forward(R, wl, shape)
         check(backward(pb, g, img, bent), other)
+
+
+@pytest.mark.parametrize("bad", BAD[:2])
+@pytest.mark.parametrize("shape", SHAPES)
+def test_gradients_of_gaussians_that_no_spoilt_pixel_blends(R, shape, bad):
+    """Lists of several batches: a pixel that has met a bad colour keeps its spoilt sums to the entries it blends, in the
+    batches in front of that colour's too."""
+    wl, clear = crowd(n=9000)
+    up = upstream(wl, 1, alpha_w=0.3)
+    seen = np.setdiff1d(np.arange(wl.scene.n), clear)[::1000]
+    colors = wl.scene.colors.copy()
+    wl.scene.colors[:] = 0.0
+    wl.scene.colors[seen] = 1.0
+    spoilt = (forward(R, wl, shape)[2]["rgb"] > 0).any(1, keepdim=True).float().expand(1, 3, -1, -1).contiguous()
+    wl.scene.colors[:] = colors
+    wl.scene.colors[seen] = 0.0
+    pb, g, img = forward(R, wl, shape)
+    assert int(pb.workspace()["tile_ranges"].diff(dim=1).max()) > 600
+    others = backward(pb, g, img, (spoilt, None, None))["colors"][:, 1] == 0
+    others[clear] = True
+    assert 0.05 < others.mean() < 0.95 and 0.005 < float(spoilt.mean()) < 0.6
+    grads = backward(pb, g, img, up)
+    wl.scene.colors[seen] = np.float32(bad)
+    pb, g, img = forward(R, wl, shape)
+    got = backward(pb, g, img, up)
+    for k in FIELDS:
+        assert np.isfinite(got[k][others]).all(), k
+        assert np.abs(got[k] - grads[k])[others].max() <= 1e-4 * np.abs(grads[k]).max(), k
