@@ -102,31 +102,32 @@ __global__ void __launch_bounds__(kCsThreads) k_scan_chunks(BinArgs a) {
 // another tile in its place goes to the counter itself) and every tile in the table takes one atomic.  An item does
 // so where an eighth of its first keys have the tile of the key 16 lanes on, or where some tile is known to hold more
 // than kEtHot keys: always, it costs latency that short problems cannot hide (a 500 k room's binning 67 -> 70 us).
-// Views of at most kEtPile Gaussians do not ask (25 us at the worst).  Binning of a 640 x 480 view, us, one atomic a
+// (32 registers, so that it does not lower the resident CTAs: 32 views 518 us at 40 registers, 511 at 32, as without.)
+// Views of at most kPile Gaussians do without (25 us at the worst).  Binning of a 640 x 480 view, us, one atomic a
 // key / counted first: 400 k Gaussians in 4 tiles 323 / 145, 2 M 1307 / 412; 2 M in 36 tiles 771 / 526.
 constexpr int kEtThreads = 128, kEtBatch = 4;
 constexpr int kEtTableBits = 9, kEtTable = 1 << kEtTableBits;
 constexpr int kEtShared = kEtThreads / 8;
 constexpr uint32_t kEtHot = 4096;
-constexpr long long kEtPile = 16384;
+constexpr long long kPile = 16384;
 constexpr uint32_t kNoTile = 0xffffffffu;
 static_assert(kChunk == 2 * kEtThreads, "two pairs per thread");
 
-__global__ void __launch_bounds__(kEtThreads) k_emit_tiles(BinArgs a) {
+template <bool PILES>
+__global__ void __launch_bounds__(kEtThreads, 16) k_emit_tiles(BinArgs a) {
     __shared__ uint32_t s_inc[kChunk];    // keys of the chunk's pairs up to and including each
     __shared__ uint32_t s_g0[kChunk];     // global tile of the rectangle's top-left corner
     __shared__ uint32_t s_wr[kChunk];     // rectangle width
     __shared__ uint32_t s_z[kChunk];      // depth bits
     __shared__ uint32_t s_wsum[kEtThreads / 32];
-    __shared__ uint32_t s_tile[kEtTable], s_cnt[kEtTable];   // tiles of a batch and its keys in them
+    __shared__ uint32_t s_tile[PILES ? kEtTable : 1], s_cnt[PILES ? kEtTable : 1];   // tiles of a batch and its keys in them
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const bool piles = a.max_count > kEtPile;
     const long long nextra =
         (long long)blockIdx.x < a.chunks ? 0 : (long long)min(a.st->ctr[kCtrEmitExtra], a.extra_cap);
     for (long long q = (long long)blockIdx.x - a.chunks; q < 0 || q < nextra; q += gridDim.x - a.chunks) {
         const uint2 it = q < 0 ? make_uint2(blockIdx.x, 0u) : a.extra[q];
         const uint4 b = a.blk[it.x];
-        const bool hot = piles && ld_relaxed_u32(a.coop + kCoopHot) != 0u;
+        const bool hot = PILES && ld_relaxed_u32(a.coop + kCoopHot) != 0u;
         const int v = blk_view(b.y);
         const ViewEntry ve = a.views[v];
         const long long local = ((long long)it.x - ve.chunk_off) * kChunk;
@@ -210,18 +211,18 @@ __global__ void __launch_bounds__(kEtThreads) k_emit_tiles(BinArgs a) {
                 }
                 p[k] = li;
             }
-            if (mb == lo && piles) {
+            if (PILES && mb == lo) {
                 const uint32_t near = __shfl_xor_sync(0xffffffffu, g[0], 16);
                 // (counted, so that every thread decides alike although each has read the note by itself)
                 few = __syncthreads_count(hot || (g[0] != kNoTile && near == g[0])) >= kEtShared;
             }
-            if (!few) {
+            if (!PILES || !few) {
 #pragma unroll
                 for (int k = 0; k < kEtBatch; ++k)
                     if (g[k] != kNoTile) rank[k] = atomicAdd(a.tile_cnt + g[k], 1u);
 #pragma unroll
                 for (int k = 0; k < kEtBatch; ++k)
-                    if (g[k] != kNoTile && rank[k] == kEtHot) st_relaxed_u32(a.coop + kCoopHot, 1u);
+                    if (PILES && g[k] != kNoTile && rank[k] == kEtHot) st_relaxed_u32(a.coop + kCoopHot, 1u);
             } else {
                 int at[kEtBatch];
                 for (int i = tid; i < kEtTable; i += kEtThreads) {
@@ -940,9 +941,10 @@ static int launch_tile_sort(BinArgs a, cudaStream_t s) {
         }))
         return GS_ERR_CUDA;
     constexpr int kWarps = THREADS / 32;
-    // a view's Gaussians bound its lists; CTAs beyond the lists share them
+    // a view's Gaussians bound its lists; CTAs beyond the lists are there to share them (a 10 k cloud over 300
+    // tiles, where nothing is shared: 41.5 us for the binning, 44 us with them)
     a.long_blocks = a.max_count > kWarpSort ? (long long)device_sm_count() * (1024 / THREADS) : 0;
-    if (a.max_count <= kCoopMin) a.long_blocks = std::min(a.long_blocks, a.G);
+    if (a.max_count <= kPile) a.long_blocks = std::min(a.long_blocks, a.G);
     k_tile_sort<THREADS><<<(unsigned)(a.long_blocks + (a.G + kWarps - 1) / kWarps), THREADS, kTileSortSmem<THREADS>, s>>>(a);
     return GS_OK;
 }
@@ -956,7 +958,9 @@ static int run_tile_first(BinArgs a, cudaStream_t s) {
     a.emit_keys = a.chunks < 8 * sms ? kEmitKeysMin : 4096u;
     if (a.chunks > 0) {
         launch_scan_chunks(a, false, s);
-        k_emit_tiles<<<(unsigned)(a.chunks + 4 * sms), kEtThreads, 0, s>>>(a);
+        const unsigned grid = (unsigned)(a.chunks + 4 * sms);
+        if (a.max_count > kPile) k_emit_tiles<true><<<grid, kEtThreads, 0, s>>>(a);
+        else k_emit_tiles<false><<<grid, kEtThreads, 0, s>>>(a);
         count_launches(1);
     } else if (cudaMemsetAsync(&a.st->num_keys, 0, sizeof(unsigned long long), s) != cudaSuccess ||
                cudaMemsetAsync(a.st->claim_cnt, 0, sizeof(uint32_t) * kClaimClasses, s) != cudaSuccess) {
