@@ -270,9 +270,10 @@ constexpr int kResident = (kWide<TW, TH, NB> ? 2048 : 2560) / (TW * TH);
 // they are only while the entry's colour and depth and the pixel's upstream gradient are tame: 0 x NaN is NaN, and a
 // lane whose quarter has no entry left reads another entry of the batch.  The projection gives other entries an
 // infinite cut-off, and their batches (and, in the backward, those of a tile with other gradients) take the SLOW
-// walk, in which a pixel's sums meet only the entries that it blends.  The backward of short lists looks at the
-// gradients once a batch: a flag kept through the walk cost it 1 % (32 views, 7.3M list entries: 2119 for 2093 us).
-// That of long lists keeps the flag: a look per batch cost it 2 % (8 views, 10.7M: 2247 for 2201 us).
+// walk, in which a pixel's sums meet only the entries that it blends.  The backward of short lists looks at gradients and
+// sums once a batch: a flag kept through the walk cost it 1 % (32 views, 7.3M list entries: 2119 for 2093 us).  That of
+// long lists keeps the flag, and a tile stays with the SLOW walk once an entry has asked for it (8 views, 10.7M: 2247 us
+// with a look per batch, 2236 with a look after each SLOW walk, 2212 so, 2203 without any of this).
 __device__ __forceinline__ float2 select2(bool x, bool y, float2 a, float2 b) {
     return make_float2(x ? a.x : b.x, y ? a.y : b.y);
 }
@@ -347,8 +348,8 @@ __global__ void __launch_bounds__(TW *TH / kPPT, kResident<TW, TH, NB>) k_render
         uint32_t bdone = __ballot_sync(0xffffffffu, done[0] && done[1]);
         bool qdone = ((bdone >> (lane & 24)) & 255u) == 255u;
         // one batch's entries, front to back; SLOW: see stage_masks
-        auto walk = [&](auto slow, const float4 *rec, const uint32_t *msk, int b, int cnt) {
-            constexpr bool SLOW = decltype(slow)::value;
+        auto walk = [&](auto is_slow, const float4 *rec, const uint32_t *msk, int b, int cnt) {
+            constexpr bool SLOW = decltype(is_slow)::value;
             for (int k0 = 0; k0 < cnt; k0 += 32) {
                 const int kk = k0 + lane;
                 uint32_t bits = quarter_bits<TW>(kk < cnt ? msk[kk] : 0u, cell0, lane);
@@ -623,17 +624,17 @@ __global__ void __launch_bounds__(TW *TH / kPPT, kResident<TW, TH, NB>) k_render
         const float2 py = make_float2((float)y0 + 0.5f, (float)(y0 + 1) + 0.5f);
         const int wmax = __reduce_max_sync(0xffffffffu, tmax);
         if (lane == 0) atomicMax(&sm.maxlast, wmax);
-        bool bent = false;                 // (kWide) the warp's gradients or sums are not tame
-        if constexpr (kWide<TW, TH, NB>)
-            bent = __any_sync(0xffffffffu, !(tame(tC0[0], tC1[0], tC2[0], tD[0]) && tame(tC0[1], tC1[1], tC2[1], tD[1]) &&
-                                             tame(tQ[0], tQ[1], 0.f, 0.f)));
+        // (kWide) an upstream gradient of this thread is not tame; from the first batch on, of the tile, or an entry
+        // so far asked for the SLOW walk (which may have spoilt a sum)
+        bool slow = kWide<TW, TH, NB> && !(tame(tC0[0], tC1[0], tC2[0], tD[0]) && tame(tC0[1], tC1[1], tC2[1], tD[1]) &&
+                                           tame(tQ[0], tQ[1], 0.f, 0.f));
         // the quarter's largest last index
         int qmax = tmax;
 #pragma unroll
         for (int o = 4; o > 0; o >>= 1) qmax = max(qmax, __shfl_xor_sync(0xffffffffu, qmax, o));
         // one batch's entries (positions lo on), back to front; SLOW: see stage_masks
-        auto walk = [&](auto slow, const float4 *rec, const uint32_t *msk, int lo, int kend) {
-            constexpr bool SLOW = decltype(slow)::value;
+        auto walk = [&](auto is_slow, const float4 *rec, const uint32_t *msk, int lo, int kend) {
+            constexpr bool SLOW = decltype(is_slow)::value;
             for (int k0 = ((kend - 1) >> 5) << 5; k0 >= 0 && kend > 0; k0 -= 32) {
                 const int kk = k0 + lane;
                 uint32_t bits = quarter_bits<TW>(kk < kend ? msk[kk] : 0u, cell0, lane);
@@ -773,18 +774,13 @@ __global__ void __launch_bounds__(TW *TH / kPPT, kResident<TW, TH, NB>) k_render
             }
             parity[buf] ^= 1u;
             const float4 *rec = sm.rec[buf];
-            bool calm = true;
             if constexpr (!kWide<TW, TH, NB>)
-                calm = tame(gC0.x, gC1.x, gC2.x, gD.x) && tame(gC0.y, gC1.y, gC2.y, gD.y) && tame(Q.x, Q.y, 0.f, 0.f);
-            const bool slow = __syncthreads_or(stage_masks<TW, TH, NB>(rec, sm.mask, cnt, tx * TW, ty * TH) | !calm);
+                slow = !(tame(gC0.x, gC1.x, gC2.x, gD.x) && tame(gC0.y, gC1.y, gC2.y, gD.y) && tame(Q.x, Q.y, 0.f, 0.f));
+            slow = __syncthreads_or(stage_masks<TW, TH, NB>(rec, sm.mask, cnt, tx * TW, ty * TH) | slow);
             // entries at or beyond the warp's largest last_idx contribute nothing to this warp
             const int kend = min(hi, wmax) - lo;
-            if (slow || bent) {
-                walk(std::true_type(), rec, sm.mask, lo, kend);
-                if constexpr (kWide<TW, TH, NB>) bent = bent || __any_sync(0xffffffffu, !tame(Q.x, Q.y, 0.f, 0.f));
-            } else {
-                walk(std::false_type(), rec, sm.mask, lo, kend);
-            }
+            if (slow) walk(std::true_type(), rec, sm.mask, lo, kend);
+            else walk(std::false_type(), rec, sm.mask, lo, kend);
             __syncthreads();                          // buffer reads finished before its refill
             buf ^= 1;
         }
